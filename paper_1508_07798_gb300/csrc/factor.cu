@@ -770,16 +770,15 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
             }
         }
         std::vector<std::vector<int>> work(maxd + 1);
-        std::vector<size_t> idsmem(maxd + 1, 0), tallsmem(maxd + 1, 0);
+        std::vector<size_t> idsmem(maxd + 1, 0);
         for (int i = 0; i < nn; ++i) {
             int dpt = ndepth[i];
             if (dpt == 0) continue;  // roots carry no basis
             int r = cfs[nodes[i].cf].r;
-            int mcap = nodes[i].s[0].mcap, kcap = nodes[i].s[0].kcap;
+            int mcap = nodes[i].s[0].mcap;
             work[dpt].push_back(2 * i);
             work[dpt].push_back(2 * i + 1);
             idsmem[dpt] = std::max(idsmem[dpt], id_smem_bytes(r, mcap, (int)sizeof(T)));
-            tallsmem[dpt] = std::max(tallsmem[dpt], sizeof(int) * (mcap + 2) + sizeof(T) * (size_t)mcap * kcap + 16);
         }
         for (int dpt = maxd; dpt >= 1; --dpt) {
             if (work[dpt].empty()) continue;
@@ -814,15 +813,22 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
             }
         }
         // ---- expansion of the finished fronts: tall bases, then H tiles
+        int kmax_tall = 0;
+        for (int c = 0; c < nc; ++c)
+            if (done[c] && !dense[c]) kmax_tall = std::max(kmax_tall, hfk[c]);
         for (int dpt = maxd; dpt >= 1; --dpt) {
-            std::vector<int> wk;
-            for (int x : work[dpt])
-                if (done[nodes[x >> 1].cf] && !dense[nodes[x >> 1].cf]) wk.push_back(x);
+            std::vector<TallItem> wk;
+            for (int x : work[dpt]) {
+                const NodeDev &N = nodes[x >> 1];
+                if (!done[N.cf] || dense[N.cf]) continue;
+                const int R = N.hi - N.lo, Ra = N.a < 0 ? R : nodes[N.a].hi - nodes[N.a].lo;
+                for (int r0 = 0; r0 < Ra; r0 += TALL_ROWS) wk.push_back({x, r0, Ra});
+                for (int r0 = Ra; r0 < R; r0 += TALL_ROWS) wk.push_back({x, r0, R});
+            }
             if (wk.empty()) continue;
-            int *d_wk;
+            TallItem *d_wk;
             if ((rc = W.up(wk, &d_wk))) return rc;
-            if ((rc = launch_hss_tall<T>(d_nodes, d_wk, (int)wk.size(), d_kout, ws, d_iws, tallsmem[dpt], s)))
-                return rc;
+            if ((rc = launch_hss_tall<T>(d_nodes, d_wk, (int)wk.size(), d_kout, ws, d_iws, kmax_tall, s))) return rc;
         }
         std::vector<ExpandItem> items;
         int kmax_done = 0;

@@ -452,55 +452,100 @@ __global__ void __launch_bounds__(ID_NT) k_hss_id(const NodeDev *__restrict__ no
     }
 }
 
-// Tall bases, bottom-up: U^tall (|R| x k, ld |R|) of each node side.
+// Tall bases, bottom-up: U^tall (|R| x k, ld |R|) of each node side, one CTA
+// per TALL_ROWS rows of one child's part of R (a leaf: of R).  A parent's tile
+// is the product U^tall_child (rows x kc) * U_l (kc x k): both factors are
+// staged in shared memory and every thread accumulates a 4 x TALL_CPT block in
+// registers (rows 4 (tid % 16) .. + 3, columns tid / 16 + 16 c), q ascending,
+// so a row's sums do not depend on the tiling.  One CTA per node side, one
+// output per thread and both factors read from L2 in every product, left all
+// but the node count of the SMs idle and spent two loads per FMA: Helmholtz
+// 64 x 64, p = 3, tol 1e-6 (ranks to 62), all tall bases of one factorization
+// 16.3 -> about 1.2 ms, the solve 64.0 -> 48.9 ms.
+constexpr int TALL_CPT = 8;   // columns per thread: k <= 128
+
 template <class T>
-__global__ void k_hss_tall(const NodeDev *__restrict__ nodes, const int *__restrict__ work,
-                           const int *__restrict__ kout, T *__restrict__ ws, const int *__restrict__ iws) {
+__global__ void __launch_bounds__(256) k_hss_tall(const NodeDev *__restrict__ nodes, const TallItem *__restrict__ work,
+                                                const int *__restrict__ kout, T *__restrict__ ws,
+                                                const int *__restrict__ iws) {
     pdl_launch_next();
     pdl_wait_prev();
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int node = work[blockIdx.x] >> 1, side = work[blockIdx.x] & 1;
-    const NodeDev N = nodes[node];
-    const NodeSide me = N.s[side];
+    const TallItem it = work[blockIdx.x];
+    const int node = it.x >> 1, side = it.x & 1;
+    const NodeDev &N = nodes[node];
+    const NodeSide &me = N.s[side];
     const int k = kout[2 * node + side];
+    if (k == 0) return;
     const int R = N.hi - N.lo;
     const bool leaf = N.a < 0;
-    int ka = 0, m = R;
-    if (!leaf) {
-        ka = kout[2 * N.a + side];
-        m = ka + kout[2 * N.b + side];
-    }
-    int *inv = reinterpret_cast<int *>(smraw);                          // m
-    T *Ul = reinterpret_cast<T *>(smraw + sizeof(int) * ((m + 1) & ~1)); // m x k (ld m)
     const int *ord = iws + me.ordoff;
-    for (int c = threadIdx.x; c < m; c += blockDim.x) inv[ord[c]] = c;
-    __syncthreads();
     const T *Tm = ws + me.toff;
-    for (int idx = threadIdx.x; idx < m * k; idx += blockDim.x) {
-        int q = idx % m, i = idx / m;
-        int p = inv[q];
-        Ul[q + (long)m * i] = p < k ? T(p == i ? 1 : 0) : Tm[i + (long)me.kcap * (p - k)];
-    }
-    __syncthreads();
+    const int ldt = me.kcap;
     T *out = ws + me.talloff;
+    const int nr = min(TALL_ROWS, it.row1 - it.row0);
     if (leaf) {
-        for (int idx = threadIdx.x; idx < R * k; idx += blockDim.x) out[idx] = Ul[idx];
+        // U itself: row ord[p] is e_p (p < k) or row p - k of T^t
+        for (int p = threadIdx.x & 31; p < R; p += 32) {
+            const int q = ord[p];
+            if (q < it.row0 || q >= it.row0 + nr) continue;
+            for (int i = threadIdx.x >> 5; i < k; i += 8)
+                out[q + (long)R * i] = p < k ? T(p == i ? 1 : 0) : Tm[i + (long)ldt * (p - k)];
+        }
         return;
     }
-    const NodeSide sa = nodes[N.a].s[side], sb = nodes[N.b].s[side];
-    const int Ra = nodes[N.a].hi - nodes[N.a].lo, Rb = nodes[N.b].hi - nodes[N.b].lo;
-    const int kb_ = m - ka;
-    const T *Ua = ws + sa.talloff, *Ub = ws + sb.talloff;
-    for (int idx = threadIdx.x; idx < R * k; idx += blockDim.x) {
-        int rho = idx % R, i = idx / R;
-        T acc = 0;
-        if (rho < Ra) {
-            for (int q = 0; q < ka; ++q) acc += Ua[rho + (long)Ra * q] * Ul[q + (long)m * i];
-        } else {
-            int rr = rho - Ra;
-            for (int q = 0; q < kb_; ++q) acc += Ub[rr + (long)Rb * q] * Ul[ka + q + (long)m * i];
+    const int ka = kout[2 * N.a + side], m = ka + kout[2 * N.b + side];
+    const int Ra = nodes[N.a].hi - nodes[N.a].lo;
+    const bool second = it.row0 >= Ra;
+    const NodeDev &C = nodes[second ? N.b : N.a];
+    const int q0 = second ? ka : 0, kc = second ? m - ka : ka;   // the child's rows of U_l
+    const int Rc = C.hi - C.lo, row0 = it.row0 - (second ? Ra : 0);
+    const T *Uc = ws + C.s[side].talloff;
+    T *Us = reinterpret_cast<T *>(smraw);        // TALL_ROWS x kc (ld TALL_ROWS)
+    T *Ul = Us + TALL_ROWS * kc;                 // kc x k, row q at ldu q
+    const int ldu = k | 1;
+    for (int idx = threadIdx.x; idx < TALL_ROWS * kc; idx += 256) {
+        const int rr = idx % TALL_ROWS, q = idx / TALL_ROWS;
+        Us[idx] = rr < nr ? Uc[row0 + rr + (long)Rc * q] : T(0);
+    }
+    for (int p = threadIdx.x >> 5; p < m; p += 8) {
+        const int q = ord[p] - q0;
+        if (q < 0 || q >= kc) continue;
+        for (int i = threadIdx.x & 31; i < k; i += 32)
+            Ul[q * ldu + i] = p < k ? T(p == i ? 1 : 0) : Tm[i + (long)ldt * (p - k)];
+    }
+    __syncthreads();
+    const int tr = (threadIdx.x & 15) * 4, tc = threadIdx.x >> 4;
+    T acc[TALL_CPT][4];
+#pragma unroll
+    for (int c = 0; c < TALL_CPT; ++c)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) acc[c][a] = T(0);
+    auto run = [&](auto ncc) {
+        constexpr int NC = decltype(ncc)::value;
+        for (int q = 0; q < kc; ++q) {
+            T u[4];
+#pragma unroll
+            for (int a = 0; a < 4; a += 16 / (int)sizeof(T)) ld16(Us + TALL_ROWS * q + tr + a, u + a);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const T b = Ul[q * ldu + min(tc + 16 * c, k - 1)];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) acc[c][a] += u[a] * b;
+            }
         }
-        out[idx] = acc;
+    };
+    if (k <= 16) run(std::integral_constant<int, 1>{});
+    else if (k <= 32) run(std::integral_constant<int, 2>{});
+    else if (k <= 64) run(std::integral_constant<int, 4>{});
+    else run(std::integral_constant<int, TALL_CPT>{});
+#pragma unroll
+    for (int c = 0; c < TALL_CPT; ++c) {
+        const int i = tc + 16 * c;
+        if (i >= k) break;
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            if (tr + a < nr) out[it.row0 + tr + a + (long)R * i] = acc[c][a];
     }
 }
 
@@ -577,11 +622,13 @@ int launch_hss_id(const NodeDev *nodes, const int *work, int nwork, const CompFr
 }
 
 template <class T>
-int launch_hss_tall(const NodeDev *nodes, const int *work, int nwork, const int *kout, T *ws, int *iws, size_t smem,
+int launch_hss_tall(const NodeDev *nodes, const TallItem *work, int nwork, const int *kout, T *ws, int *iws, int kmax,
                     cudaStream_t s) {
     if (nwork == 0) return HSS_OK;
     HSS_SMEM(k_hss_tall<T>, 220 * 1024);
     HSS_PROF("hss_tall", s);
+    // a child's rows of U_l (kmax x kmax, odd leading dimension) and its tile of U^tall
+    const size_t smem = sizeof(T) * ((size_t)kmax * (kmax | 1) + (size_t)TALL_ROWS * kmax) + 16;
     HSS_CUDA(launch_pdl(k_hss_tall<T>, dim3(nwork), dim3(256), smem, s, nodes, work, kout, ws, (const int *)iws));
     HSS_CHECK_LAUNCH("k_hss_tall");
     return HSS_OK;
@@ -720,7 +767,7 @@ int launch_hss_probe(const ProbeItem *items, int nitems, const ProbeFront *pf, i
                                      const T *, uint64_t, int, double *, double *, cudaStream_t);               \
     template int launch_hss_id<T>(const NodeDev *, const int *, int, const CompFront<T> *, T *, int *, int *,  \
                                   int *, T, uint64_t, size_t, cudaStream_t);                                  \
-    template int launch_hss_tall<T>(const NodeDev *, const int *, int, const int *, T *, int *, size_t,        \
+    template int launch_hss_tall<T>(const NodeDev *, const TallItem *, int, const int *, T *, int *, int,      \
                                     cudaStream_t);                                                             \
     template int launch_hss_expand<T>(const ExpandItem *, int, const NodeDev *, const int *, const ExpandFront *, \
                                       const T *, const int *, T *, T *, int, cudaStream_t);

@@ -52,6 +52,13 @@ struct NodeDev {
     NodeSide s[2];
 };
 
+// Rows [row0, min(row1, row0 + TALL_ROWS)) of the tall basis of a node side
+// (x = 2 node + side); row1 ends the child's part of the node's rows.
+constexpr int TALL_ROWS = 64;
+struct TallItem {
+    int x, row0, row1;
+};
+
 // One 32 x 32 tile of the expanded approximant H written into the parent front.
 struct ExpandItem {
     int type;         // 0: copy S block (leaf diagonal block / whole S); 1: U^tall_a S(J_a,K_b) V^tall_b^t
@@ -92,8 +99,8 @@ template <class T>
 int launch_hss_id(const NodeDev *nodes, const int *work, int nwork, const CompFront<T> *cf, T *ws, int *iws,
                   int *kout, int *front_kmax, T tol, uint64_t seed, size_t smem, cudaStream_t s);
 template <class T>
-int launch_hss_tall(const NodeDev *nodes, const int *work, int nwork, const int *kout, T *ws, int *iws, size_t smem,
-                    cudaStream_t s);
+int launch_hss_tall(const NodeDev *nodes, const TallItem *work, int nwork, const int *kout, T *ws, int *iws, int kmax,
+                    cudaStream_t s);   // kmax: largest rank of the work's nodes and their children
 template <class T>
 int launch_hss_expand(const ExpandItem *items, int nitems, const NodeDev *nodes, const int *kout,
                       const ExpandFront *ef, const T *ws, const int *iws, T *arena, T *keep, int kmax,
