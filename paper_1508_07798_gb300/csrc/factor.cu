@@ -652,6 +652,8 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
             cfs[c].nb = d.nb;
             cfs[c].r = r;
             cfs[c].box = key_of(active[c].f);
+            // (the rule applied to the ranks read back below)
+            cfs[c].k_again = r < d.nb && r + o.dr <= o.rmax ? r - o.oversample : INT32_MAX;
             cfs[c].yoff = wsz;
             wsz += (long)d.nb * r;
             cfs[c].zoff = wsz;
@@ -770,24 +772,56 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
             }
         }
         std::vector<std::vector<int>> work(maxd + 1);
-        std::vector<size_t> idsmem(maxd + 1, 0);
         for (int i = 0; i < nn; ++i) {
             int dpt = ndepth[i];
             if (dpt == 0) continue;  // roots carry no basis
-            int r = cfs[nodes[i].cf].r;
-            int mcap = nodes[i].s[0].mcap;
             work[dpt].push_back(2 * i);
             work[dpt].push_back(2 * i + 1);
-            idsmem[dpt] = std::max(idsmem[dpt], id_smem_bytes(r, mcap, (int)sizeof(T)));
         }
+        // the node sides of a depth by register form of the ID (hss.h): all in the
+        // form that holds the largest of them, or, beyond two per SM, one launch
+        // per form, so that small nodes do not occupy the threads of large ones.
+        // One upload serves every launch (a copy between two of them would keep
+        // the second from being set up while the first runs).
+        struct IdLaunch {
+            int off, cnt, r, m, key;
+            size_t smem;
+        };
+        std::vector<IdLaunch> ids;
+        std::vector<int> id_work;
         for (int dpt = maxd; dpt >= 1; --dpt) {
-            if (work[dpt].empty()) continue;
-            int *d_work;
-            if ((rc = W.up(work[dpt], &d_work))) return rc;
-            if ((rc = launch_hss_id<T>(d_nodes, d_work, (int)work[dpt].size(), d_cfs, ws, d_iws, d_kout, d_fk,
-                                       (T)o.tol, o.seed, idsmem[dpt], s)))
-                return rc;
+            const bool split = (int)work[dpt].size() > 2 * device_sms();
+            std::vector<int> cls(work[dpt].size(), 0);
+            for (size_t i = 0; i < work[dpt].size() && split; ++i) {
+                const NodeDev &N = nodes[work[dpt][i] >> 1];
+                const IdClass ic = id_class(cfs[N.cf].r, N.s[0].mcap, (int)sizeof(T));
+                cls[i] = ic.r * 1024 + ic.m;
+            }
+            std::vector<int> keys(cls);
+            std::sort(keys.begin(), keys.end());
+            keys.erase(std::unique(keys.begin(), keys.end()), keys.end());
+            for (int key : keys) {
+                IdLaunch L{(int)id_work.size(), 0, 0, 0, key, 0};
+                for (size_t i = 0; i < work[dpt].size(); ++i) {
+                    if (cls[i] != key) continue;
+                    const NodeDev &N = nodes[work[dpt][i] >> 1];
+                    const int r = cfs[N.cf].r, m = N.s[0].mcap;
+                    id_work.push_back(work[dpt][i]);
+                    L.r = std::max(L.r, r);
+                    L.m = std::max(L.m, m);
+                }
+                const IdClass ic = id_class(L.r, L.m, (int)sizeof(T));
+                L.smem = id_smem_bytes(std::max(L.r, ic.r), L.m, (int)sizeof(T));   // a register form's R has its largest r
+                L.cnt = (int)id_work.size() - L.off;
+                ids.push_back(L);
+            }
         }
+        int *d_work;
+        if ((rc = W.up(id_work, &d_work))) return rc;
+        for (const IdLaunch &L : ids)
+            if ((rc = launch_hss_id<T>(d_nodes, d_work + L.off, L.cnt, L.r, L.m, d_cfs, ws, d_iws, d_kout, d_fk, (T)o.tol,
+                                       o.seed, L.smem, s)))
+                return rc;
         std::vector<int> hfk(nc);
         if ((rc = factor_readback(hfk.data(), d_fk, sizeof(int) * nc, s, F))) return rc;
         // ---- decide: fronts whose rank reached r - oversample sample again, wider
@@ -816,8 +850,10 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
         int kmax_tall = 0;
         for (int c = 0; c < nc; ++c)
             if (done[c] && !dense[c]) kmax_tall = std::max(kmax_tall, hfk[c]);
+        std::vector<TallItem> wk;
+        std::vector<int> wk_off;   // per depth, deepest first
         for (int dpt = maxd; dpt >= 1; --dpt) {
-            std::vector<TallItem> wk;
+            wk_off.push_back((int)wk.size());
             for (int x : work[dpt]) {
                 const NodeDev &N = nodes[x >> 1];
                 if (!done[N.cf] || dense[N.cf]) continue;
@@ -825,10 +861,15 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
                 for (int r0 = 0; r0 < Ra; r0 += TALL_ROWS) wk.push_back({x, r0, Ra});
                 for (int r0 = Ra; r0 < R; r0 += TALL_ROWS) wk.push_back({x, r0, R});
             }
-            if (wk.empty()) continue;
+        }
+        wk_off.push_back((int)wk.size());
+        if (!wk.empty()) {
             TallItem *d_wk;
             if ((rc = W.up(wk, &d_wk))) return rc;
-            if ((rc = launch_hss_tall<T>(d_nodes, d_wk, (int)wk.size(), d_kout, ws, d_iws, kmax_tall, s))) return rc;
+            for (size_t q = 0; q + 1 < wk_off.size(); ++q)
+                if ((rc = launch_hss_tall<T>(d_nodes, d_wk + wk_off[q], wk_off[q + 1] - wk_off[q], d_kout, ws, d_iws,
+                                             kmax_tall, s)))
+                    return rc;
         }
         std::vector<ExpandItem> items;
         int kmax_done = 0;

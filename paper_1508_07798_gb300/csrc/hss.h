@@ -23,6 +23,22 @@ inline size_t id_smem_bytes(int r, int mcap, int esize) {
     return (size_t)esize * ((size_t)id_lda(r, esize) * mcap + r + mcap) + sizeof(int) * (size_t)mcap + 16;
 }
 
+// Register forms of the FP32 ID kernel: node sides with sample width <= r and
+// at most m columns (r = 0: the general form).  {32, 64}, {64, 64 / 128},
+// {96, 64 / 128 / 192}: a parent has at most two children of rank <= r.  FP64
+// keeps the general form: its ID is bound by the FP64 pipe (measured on the
+// 64 x 64, p = 2 Helmholtz factorization: 15.8 ms in both forms).
+struct IdClass {
+    int r, m;
+};
+inline IdClass id_class(int r, int m, int esize) {
+    if (r > 96 || m > 192 || esize != 4) return {0, 0};
+    const int rc = r <= 32 ? 32 : r <= 64 ? 64 : 96, mc = m <= 64 ? 64 : m <= 128 ? 128 : 192;
+    if (rc == 32 && mc > 64) return id_class(33, m, esize);
+    if (rc == 64 && mc > 128) return id_class(65, m, esize);
+    return {rc, mc};
+}
+
 // A front being compressed in the current sampling round.
 template <class T> struct CompFront {
     const T *S;       // Schur complement inside the front (column-major)
@@ -30,6 +46,7 @@ template <class T> struct CompFront {
     int nb;           // order of S
     int r;            // sample width of the current sampling round
     int box;          // front id of the test-matrix counter
+    int k_again;      // a node rank above this sends the front to a wider sampling round
     long yoff, zoff;  // samples Y = S Omega, Z = S^t Psi (nb x r, ld nb) in the sample buffer
 };
 
@@ -96,8 +113,9 @@ struct ProbeFront {
 };
 
 template <class T>
-int launch_hss_id(const NodeDev *nodes, const int *work, int nwork, const CompFront<T> *cf, T *ws, int *iws,
-                  int *kout, int *front_kmax, T tol, uint64_t seed, size_t smem, cudaStream_t s);
+int launch_hss_id(const NodeDev *nodes, const int *work, int nwork, int rmax, int mmax, const CompFront<T> *cf, T *ws,
+                  int *iws, int *kout, int *front_kmax, T tol, uint64_t seed, size_t smem, cudaStream_t s);   // rmax,
+                  // mmax: largest sample width and column count of the work
 template <class T>
 int launch_hss_tall(const NodeDev *nodes, const TallItem *work, int nwork, const int *kout, T *ws, int *iws, int kmax,
                     cudaStream_t s);   // kmax: largest rank of the work's nodes and their children
