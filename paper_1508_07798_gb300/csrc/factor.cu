@@ -385,8 +385,9 @@ int eliminate_stage(const std::vector<FrontDev> &fr, const FrontDev *d_fr, T *ar
             }
         // tall fronts: 32-column panels spread over a cluster while their rows
         // exceed one CTA's registers, then the register panel
-        if (fr[f].ni > PANEL_CL_MIN_NI && panel_cl_fits(PANEL_KB_MAX, fr[f].ni, (int)sizeof(T))) {
+        if (fr[f].ni > (sizeof(T) == 4 ? PANEL_CL_MIN_NI_F32 : PANEL_CL_MIN_NI) && panel_cl_fits(PANEL_KB_MAX, fr[f].ni, (int)sizeof(T))) {
             kb[f] = PANEL_KB_MAX;
+            isreg[f] = 0;
             clpath[f] = 1;
         }
         Rf[f] = cdiv(std::max(fr[f].ni, 1), PANEL_NT);

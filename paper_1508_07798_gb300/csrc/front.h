@@ -84,7 +84,13 @@ bool panel_cl_fits(int kb, int rows, int tsize);
 // rows a cluster panel of `rows` rows is launched for (its shape's capacity);
 // jobs of one launch share it
 int panel_cl_capacity(int rows, int tsize);
-constexpr int PANEL_CL_MIN_NI = 6144;   // fronts with more interior dofs take the cluster panel
+// Fronts with more interior dofs take the cluster panel.  FP32: where 32-column
+// panels leave one CTA's registers; the narrower register panels beyond took 2 to
+// 4 times the panel, post-panel and update launches and blocks of 128 or 64
+// columns (a 6,000-row front with 4,000 interior dofs: panels 8.6 -> 7.8, post
+// 5.0 -> 1.7, in-block updates 4.2 -> 1.6, block updates 8.2 -> 1.5 ms).
+// FP64: beyond 6,144, where the register panels end.
+constexpr int PANEL_CL_MIN_NI = 6144, PANEL_CL_MIN_NI_F32 = 1536;
 template <class T>
 int launch_gj_panel_cl(const PanelJob *jobs, int njobs, int cap, size_t smem, const FrontDev *fr, T *arena, T *xws,
                        int *mws, int *piv, int *rperm, const int *ilist, int *iperm, int *status, cudaStream_t s,
