@@ -25,19 +25,11 @@ constexpr int AP_NT = 256;
 constexpr int AP_WPB = AP_NT / 32;   // warps (work items) per CTA
 
 
-// One warp per work item = (front, 32-row tile, column chunk of at most
-// APPLY_CHUNK columns).  Lane l owns row row0 + l; x is gathered one value per
-// lane and broadcast by shuffles; 32 matrix loads per lane are in flight per
-// group of 32 columns.  A tile split over several chunks writes partial sums;
-// the last warp to finish (atomic ticket) adds them in chunk order and writes
-// the result, so the sum order is fixed.  No barrier, no waiting.
-//   FWD: y = [F_ii^-1 P^t ; -F_bi F_ii^-1 P^t] x(Iperm)  ->  t = y[0,ni), x_B += y[ni,n)
-//   BWD: x_I = t - W x_B
-// The products of one work item: lane l's sums for row row0 + l.
-template <class T, int RB, bool FWD>
-__device__ __forceinline__ void apply_item_sums(const ApplyItem &it, const FrontDev &F, const T *__restrict__ arena,
-                                                const int *__restrict__ iperm, const int *__restrict__ blist,
-                                                const double *__restrict__ w, long ldw, int nrhs, T (&acc)[RB]) {
+// The products of one work item: lane l's sum for row row0 + l.
+template <class T, bool FWD>
+__device__ __forceinline__ T apply_item_sum(const ApplyItem &it, const FrontDev &F, const T *__restrict__ arena,
+                                            const int *__restrict__ iperm, const int *__restrict__ blist,
+                                            const double *__restrict__ w) {
     const int lane = threadIdx.x & 31;
     const T *M = arena + F.foff;
     const int colbase = FWD ? 0 : F.ni, nrows = FWD ? F.n : F.ni;
@@ -45,8 +37,7 @@ __device__ __forceinline__ void apply_item_sums(const ApplyItem &it, const Front
     const bool rowok = i < nrows;
     // arithmetic in the factor's precision (FP32 factors: FP32 products and sums;
     // GB300's FP64 pipe is a small fraction of its FP32 rate)
-#pragma unroll
-    for (int r = 0; r < RB; ++r) acc[r] = T(0);
+    T acc = T(0);
     bool waited = false;
     for (int cg = it.c0; cg < it.c1; cg += 32) {
         const int c = cg + lane;
@@ -59,50 +50,43 @@ __device__ __forceinline__ void apply_item_sums(const ApplyItem &it, const Front
             pdl_wait_prev();
             waited = true;
         }
-        T z[RB];
+        const T z = dof >= 0 ? (T)w[dof] : T(0);
 #pragma unroll
-        for (int r = 0; r < RB; ++r) z[r] = (dof >= 0 && r < nrhs) ? (T)w[dof + ldw * r] : T(0);
-#pragma unroll
-        for (int q = 0; q < 32; ++q) {
-#pragma unroll
-            for (int r = 0; r < RB; ++r) acc[r] = fma(m[q], __shfl_sync(0xffffffffu, z[r], q), acc[r]);
-        }
+        for (int q = 0; q < 32; ++q) acc = fma(m[q], __shfl_sync(0xffffffffu, z, q), acc);
     }
+    return acc;
 }
 
-// The results of one work item (row row0 + lane):
-//   FWD: rows [0, ni) to t, rows [ni, n) added into x_B;  BWD: x_I = t - sums
-template <class T, int RB, bool FWD>
+// The result of one work item (row row0 + lane):
+//   FWD: rows [0, ni) to t, rows [ni, n) added into x_B;  BWD: x_I = t - sum
+template <class T, bool FWD>
 __device__ __forceinline__ void apply_item_store(const ApplyItem &it, const FrontDev &F, const int *__restrict__ ilist,
-                                                 const int *__restrict__ blist, double *__restrict__ w, long ldw,
-                                                 double *__restrict__ tv, long ldt, int nrhs, const T (&acc)[RB]) {
+                                                 const int *__restrict__ blist, double *__restrict__ w,
+                                                 double *__restrict__ tv, T acc) {
     const int i = it.row0 + (threadIdx.x & 31);
     if (i >= (FWD ? F.n : F.ni)) return;
-#pragma unroll
-    for (int r = 0; r < RB; ++r) {
-        if (r >= nrhs) break;
-        const double y = (double)acc[r];
-        if (FWD) {
-            if (i < F.ni)
-                tv[ilist[F.iset_off + i] + ldt * r] = y;
-            else
-                w[blist[F.bset_off + i - F.ni] + ldw * r] += y;
-        } else {
-            const int dof = ilist[F.iset_off + i];
-            w[dof + ldw * r] = tv[dof + ldt * r] - y;
-        }
+    const double y = (double)acc;
+    if (FWD) {
+        if (i < F.ni)
+            tv[ilist[F.iset_off + i]] = y;
+        else
+            w[blist[F.bset_off + i - F.ni]] += y;
+    } else {
+        const int dof = ilist[F.iset_off + i];
+        w[dof] = tv[dof] - y;
     }
 }
 
-// One warp per work item = (front, 32-row tile, column chunk of at most
-// APPLY_CHUNK columns).  Lane l owns row row0 + l; x is gathered one value per
-// lane and broadcast by shuffles; 32 matrix loads per lane are in flight per
-// group of 32 columns.  A tile split over several chunks writes partial sums;
-// the last warp to finish (atomic ticket) adds them in chunk order and writes
-// the result, so the sum order is fixed.  No barrier, no waiting.
+// One vector (several: apply_multi.cu).  One warp per work item = (front,
+// 32-row tile, column chunk of at most APPLY_CHUNK columns).  Lane l owns row
+// row0 + l; x is gathered one value per lane and broadcast by shuffles; 32
+// matrix loads per lane are in flight per group of 32 columns.  A tile split
+// over several chunks writes partial sums; the last warp to finish (atomic
+// ticket) adds them in chunk order and writes the result, so the sum order is
+// fixed.  No barrier, no waiting.
 //   FWD: y = [F_ii^-1 P^t ; -F_bi F_ii^-1 P^t] x(Iperm)  ->  t = y[0,ni), x_B += y[ni,n)
 //   BWD: x_I = t - W x_B
-template <class T, int RB, bool FWD>
+template <class T, bool FWD>
 __global__ void __launch_bounds__(AP_NT) k_apply(const ApplyItem *__restrict__ items, int nitems,
                                                const FrontDev *__restrict__ fr, const T *__restrict__ arena,
                                                const int *__restrict__ iperm, const int *__restrict__ ilist,
@@ -114,29 +98,22 @@ __global__ void __launch_bounds__(AP_NT) k_apply(const ApplyItem *__restrict__ i
     if (item >= nitems) return;   // whole warps leave together
     const ApplyItem it = items[item];
     const FrontDev F = fr[it.front];
-    T acc[RB];
-    apply_item_sums<T, RB, FWD>(it, F, arena, iperm, blist, prm->w, prm->ldw, prm->nrhs, acc);
+    T acc = apply_item_sum<T, FWD>(it, F, arena, iperm, blist, prm->w);
     pdl_wait_prev();   // (an item without columns has not waited yet)
     if (it.nchunk > 1) {
-        T *mine = reinterpret_cast<T *>(part) + (long)item * 32 * RB;
-#pragma unroll
-        for (int r = 0; r < RB; ++r) mine[r * 32 + lane] = acc[r];
+        reinterpret_cast<T *>(part)[(long)item * 32 + lane] = acc;
         __threadfence();
         int ticket = 0;
         if (lane == 0) ticket = atomicAdd(&tickets[it.tile], 1);
         ticket = __shfl_sync(0xffffffffu, ticket, 0);
         if (ticket != it.nchunk - 1) return;
         __threadfence();
-        const T *first = reinterpret_cast<const T *>(part) + (long)it.first * 32 * RB;
-#pragma unroll
-        for (int r = 0; r < RB; ++r) {
-            T y = T(0);
-            for (int ch = 0; ch < it.nchunk; ++ch) y += __ldcg(first + (long)ch * 32 * RB + r * 32 + lane);
-            acc[r] = y;
-        }
+        const T *first = reinterpret_cast<const T *>(part) + (long)it.first * 32;
+        acc = T(0);
+        for (int ch = 0; ch < it.nchunk; ++ch) acc += __ldcg(first + (long)ch * 32 + lane);
         if (lane == 0) tickets[it.tile] = 0;   // ready for the next apply
     }
-    apply_item_store<T, RB, FWD>(it, F, ilist, blist, prm->w, prm->ldw, prm->tv, prm->ldt, prm->nrhs, acc);
+    apply_item_store<T, FWD>(it, F, ilist, blist, prm->w, prm->tv, acc);
 }
 
 // The deepest levels as one launch: CTA s walks the stages of subtree s (the
@@ -145,7 +122,7 @@ __global__ void __launch_bounds__(AP_NT) k_apply(const ApplyItem *__restrict__ i
 // tile, every column) and a block barrier between stages.  Subtrees hold
 // disjoint dofs (DG dofs belong to elements), so the CTAs never meet; inside
 // one, the barrier orders a stage's writes of x before the next stage's reads.
-template <class T, int RB, bool FWD>
+template <class T, bool FWD>
 __global__ void __launch_bounds__(AP_NT) k_apply_sub(const ApplyItem *__restrict__ items, const int *__restrict__ off,
                                                    int nst, const FrontDev *__restrict__ fr, const T *__restrict__ arena,
                                                    const int *__restrict__ iperm, const int *__restrict__ ilist,
@@ -154,18 +131,15 @@ __global__ void __launch_bounds__(AP_NT) k_apply_sub(const ApplyItem *__restrict
     const int sub = blockIdx.x, warp = threadIdx.x >> 5;
     double *w = prm->w;
     double *tv = prm->tv;
-    const long ldw = prm->ldw, ldt = prm->ldt;
-    const int nrhs = prm->nrhs;
     for (int l = 0; l < nst; ++l) {
         const int q = FWD ? l : nst - 1 - l;
         const int b = off[sub * (nst + 1) + q], e = off[sub * (nst + 1) + q + 1];
         for (int k = b + warp; k < e; k += AP_WPB) {
             const ApplyItem it = items[k];
             const FrontDev F = fr[it.front];
-            T acc[RB];
-            apply_item_sums<T, RB, FWD>(it, F, arena, iperm, blist, w, ldw, nrhs, acc);
+            const T acc = apply_item_sum<T, FWD>(it, F, arena, iperm, blist, w);
             pdl_wait_prev();
-            apply_item_store<T, RB, FWD>(it, F, ilist, blist, w, ldw, tv, ldt, nrhs, acc);
+            apply_item_store<T, FWD>(it, F, ilist, blist, w, tv, acc);
         }
         pdl_wait_prev();   // warps without items
         __syncthreads();
@@ -191,49 +165,47 @@ __global__ void k_apply_copyin(const ApplyParams *__restrict__ prm, long N) {
 
 // The whole sweep (copy-in, forward levels, top block, backward levels) as
 // one kernel sequence on stream s, each launch overlapping the previous one's
-// tail (launch_pdl); parameters come from f->d_aparams.
+// tail (launch_pdl); parameters come from f->d_aparams.  RB = 1: one vector;
+// else up to RB, every level in a launch of its own.
 template <class T, int RB> static int record_sweep(const hss_factor_t *f, cudaStream_t s, int &nk) {
     const T *arena = f->arena_ptr<T>();
     const ApplyParams *prm = f->d_aparams.as<ApplyParams>();
+    const int *iperm = f->d_iperm.as<int>(), *blist = f->tree->d_bset.as<int>();
     nk = 0;
     k_apply_copyin<<<2 * device_sms(), 256, 0, s>>>(prm, f->ndof);
     ++nk;
     cudaError_t e = cudaSuccess;
+    const int sub_nst = RB == 1 ? f->sub_nst : 0;
     auto sub = [&](bool fwd) {
-        if (f->sub_nst == 0 || e != cudaSuccess) return;
-        const int *il = f->tree->d_iset.as<int>(), *bl = f->tree->d_bset.as<int>();
-        if (fwd)
-            e = launch_pdl(k_apply_sub<T, RB, true>, dim3(f->sub_n), dim3(AP_NT), 0, s, (const ApplyItem *)f->d_sub_fwd,
-                           (const int *)f->d_sub_off_fwd, f->sub_nst, (const FrontDev *)f->d_sub_fronts, arena,
-                           (const int *)f->d_iperm.as<int>(), il, bl, prm);
-        else
-            e = launch_pdl(k_apply_sub<T, RB, false>, dim3(f->sub_n), dim3(AP_NT), 0, s, (const ApplyItem *)f->d_sub_bwd,
-                           (const int *)f->d_sub_off_bwd, f->sub_nst, (const FrontDev *)f->d_sub_fronts, arena,
-                           (const int *)f->d_iperm.as<int>(), il, bl, prm);
-        ++nk;
+        if constexpr (RB == 1) {
+            if (sub_nst == 0 || e != cudaSuccess) return;
+            e = launch_pdl(fwd ? k_apply_sub<T, true> : k_apply_sub<T, false>, dim3(f->sub_n), dim3(AP_NT), 0, s,
+                           (const ApplyItem *)(fwd ? f->d_sub_fwd : f->d_sub_bwd),
+                           (const int *)(fwd ? f->d_sub_off_fwd : f->d_sub_off_bwd), sub_nst,
+                           (const FrontDev *)f->d_sub_fronts, arena, iperm, (const int *)f->tree->d_iset.as<int>(), blist,
+                           prm);
+            ++nk;
+        }
     };
     for (int pass = 0; pass < 2; ++pass) {
         const bool fwd = pass == 0;
         if (fwd) sub(true);
         for (size_t k = 0; k < f->apply.size(); ++k) {
             const size_t q = fwd ? k : f->apply.size() - 1 - k;
-            if ((int)q < f->sub_nst) continue;   // in the subtree launch
+            if ((int)q < sub_nst) continue;   // in the subtree launch
             const ApplyStage &st = f->apply[q];
             const int *ilist = st.top ? f->d_topset.as<int>() : f->tree->d_iset.as<int>();
             const int nt = fwd ? st.nfwd : st.nbwd;
             if (nt == 0) continue;
-            const ApplyItem *itm = fwd ? st.d_fwd : st.d_bwd;
-            double *part = f->d_apart.as<double>() + (fwd ? st.part_fwd : st.part_bwd) * 32 * APPLY_RB;
-            int *tk = f->d_tickets.as<int>() + (fwd ? st.tk_fwd : st.tk_bwd);
             if (e != cudaSuccess) break;
-            if (fwd)
-                e = launch_pdl(k_apply<T, RB, true>, dim3(cdiv(nt, AP_WPB)), dim3(AP_NT), 0, s, itm, nt, (const FrontDev *)st.d_fronts,
-                               arena, (const int *)f->d_iperm.as<int>(), ilist, (const int *)f->tree->d_bset.as<int>(),
-                               prm, part, tk);
+            if constexpr (RB > 1)
+                e = launch_apply_multi<T, RB>(f, q, fwd, s);
             else
-                e = launch_pdl(k_apply<T, RB, false>, dim3(cdiv(nt, AP_WPB)), dim3(AP_NT), 0, s, itm, nt, (const FrontDev *)st.d_fronts,
-                               arena, (const int *)f->d_iperm.as<int>(), ilist, (const int *)f->tree->d_bset.as<int>(),
-                               prm, part, tk);
+                e = launch_pdl(fwd ? k_apply<T, true> : k_apply<T, false>, dim3(cdiv(nt, AP_WPB)), dim3(AP_NT), 0, s,
+                               (const ApplyItem *)(fwd ? st.d_fwd : st.d_bwd), nt, (const FrontDev *)st.d_fronts, arena,
+                               iperm, ilist, blist, prm,
+                               f->d_apart.as<double>() + (fwd ? st.part_fwd : st.part_bwd) * 32,
+                               f->d_tickets.as<int>() + (fwd ? st.tk_fwd : st.tk_bwd));
             ++nk;
         }
         if (!fwd) sub(false);
@@ -382,7 +354,7 @@ int pack_apply(hss_factor_t *F, cudaStream_t s) {
         F->d_sub_off_bwd = reinterpret_cast<int *>(put(soff[1].data(), sizeof(int) * soff[1].size()));
     }
     HSS_CUDA(cudaMemcpyAsync(base, pack.data(), pack.size(), cudaMemcpyHostToDevice, s));
-    if ((rc = F->d_apart.alloc(sizeof(double) * 32 * APPLY_RB * std::max(part_total, 1L))) ||
+    if ((rc = F->d_apart.alloc(sizeof(double) * 32 * std::max(part_total, 1L))) ||
         (rc = F->d_tickets.alloc(sizeof(int) * std::max(tk_total, 1))))
         return rc;
     HSS_CUDA(cudaMemsetAsync(F->d_tickets.p, 0, sizeof(int) * std::max(tk_total, 1), s));
@@ -406,15 +378,15 @@ template <class T> static int timed_sweep(const hss_factor_t *f, cudaStream_t s,
             const int nt = fwd ? st.nfwd : st.nbwd;
             if (nt == 0) continue;
             const int *ilist = st.top ? f->d_topset.as<int>() : f->tree->d_iset.as<int>();
-            double *part = f->d_apart.as<double>() + (fwd ? st.part_fwd : st.part_bwd) * 32 * APPLY_RB;
+            double *part = f->d_apart.as<double>() + (fwd ? st.part_fwd : st.part_bwd) * 32;
             int *tk = f->d_tickets.as<int>() + (fwd ? st.tk_fwd : st.tk_bwd);
             HSS_CUDA(cudaEventRecord(ev[2 * (2 * q + pass)], s));
             if (fwd)
-                k_apply<T, 1, true><<<cdiv(nt, AP_WPB), AP_NT, 0, s>>>(st.d_fwd, nt, st.d_fronts, arena,
+                k_apply<T, true><<<cdiv(nt, AP_WPB), AP_NT, 0, s>>>(st.d_fwd, nt, st.d_fronts, arena,
                                                                        f->d_iperm.as<int>(), ilist,
                                                                        f->tree->d_bset.as<int>(), prm, part, tk);
             else
-                k_apply<T, 1, false><<<cdiv(nt, AP_WPB), AP_NT, 0, s>>>(st.d_bwd, nt, st.d_fronts, arena,
+                k_apply<T, false><<<cdiv(nt, AP_WPB), AP_NT, 0, s>>>(st.d_bwd, nt, st.d_fronts, arena,
                                                                         f->d_iperm.as<int>(), ilist,
                                                                         f->tree->d_bset.as<int>(), prm, part, tk);
             HSS_CUDA(cudaEventRecord(ev[2 * (2 * q + pass) + 1], s));
@@ -469,7 +441,7 @@ int tune_apply(hss_factor_t *F, cudaStream_t s) {
     if (all_known) return pack_apply(F, s);
     int rc;
     DevBuf yb;
-    if ((rc = F->tvec.alloc(sizeof(double) * (size_t)F->ndof * APPLY_RB)) ||
+    if ((rc = F->tvec.alloc(sizeof(double) * (size_t)F->ndof)) ||
         (rc = F->d_aparams.alloc(sizeof(ApplyParams))) || (rc = yb.alloc(sizeof(double) * (size_t)F->ndof)))
         return rc;
     HSS_CUDA(cudaMemsetAsync(yb.p, 0, sizeof(double) * F->ndof, s));
@@ -519,7 +491,10 @@ template <class T> static int build_graph(hss_factor_t *f, int slot) {
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         int nk = 0;
-        rc = slot == 0 ? record_sweep<T, 1>(f, cs, nk) : record_sweep<T, APPLY_RB>(f, cs, nk);
+        rc = slot == 0   ? record_sweep<T, 1>(f, cs, nk)
+             : slot == 1 ? record_sweep<T, 8>(f, cs, nk)
+             : slot == 2 ? record_sweep<T, 16>(f, cs, nk)
+                         : record_sweep<T, 32>(f, cs, nk);
         e = cudaStreamEndCapture(cs, &g);
         f->graph_kernels[slot] = nk;
     }
@@ -537,15 +512,18 @@ int apply_factor(const hss_factor_t *f, int nrhs, const double *x, long ldx, dou
     int rc;
     if ((rc = mf->tvec.alloc(sizeof(double) * (size_t)f->ndof * std::min(nrhs, APPLY_RB)))) return rc;
     if ((rc = mf->d_aparams.alloc(sizeof(ApplyParams)))) return rc;
-    const int slot = nrhs == 1 ? 0 : 1;
-    if (!f->gexec[slot]) {
-        rc = f->precision == HSS_FP32 ? build_graph<float>(mf, slot) : build_graph<double>(mf, slot);
+    if (nrhs > 1 && f->multi.empty()) {
+        rc = f->precision == HSS_FP32 ? pack_apply_multi<float>(mf, s) : pack_apply_multi<double>(mf, s);
         if (rc) return rc;
     }
     HSS_PROF("apply", s, f->apply_bytes(nrhs));
     for (int k = 0; k < nrhs; k += APPLY_RB) {   // one sweep per block of up to APPLY_RB right-hand sides
-        ApplyParams pv{x + ldx * k, ldx, y + ldy * k, ldy, mf->tvec.as<double>(), (long)f->ndof,
-                       std::min(APPLY_RB, nrhs - k)};
+        const int nr = std::min(APPLY_RB, nrhs - k), slot = nr == 1 ? 0 : nr <= 8 ? 1 : nr <= 16 ? 2 : 3;
+        if (!f->gexec[slot]) {
+            rc = f->precision == HSS_FP32 ? build_graph<float>(mf, slot) : build_graph<double>(mf, slot);
+            if (rc) return rc;
+        }
+        ApplyParams pv{x + ldx * k, ldx, y + ldy * k, ldy, mf->tvec.as<double>(), (long)f->ndof, nr};
         prof_add_launches(f->graph_kernels[slot]);
         k_apply_set<<<1, 32, 0, s>>>(mf->d_aparams.as<ApplyParams>(), pv);
         HSS_CHECK_LAUNCH("k_apply_set");

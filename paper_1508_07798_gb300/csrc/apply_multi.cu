@@ -1,0 +1,283 @@
+// The sweeps of hss_apply for several right-hand sides: each front block times
+// a block of up to 32 vectors, as a tiled product.
+//
+// A CTA takes one item = (front, 128 rows, a range of columns).  The factor's
+// columns and the gathered vector values arrive in shared memory in chunks of
+// MKC columns (the factor's by cp.async, double-buffered), and every thread
+// keeps an 8 x 4, 4 x 4 or 4 x 2 block of (row, vector) sums in registers, so a
+// factor entry is read once from HBM for all vectors of the sweep and a vector
+// value once per 128 rows.  The kernel for one vector broadcasts x by shuffles,
+// one per product: with 8 vectors it was bound by the shuffle rate, a quarter
+// of the FMA rate, read the factor again for every 8 and gathered x for every
+// 32 rows.  Sums run over the columns of an item in order and over the items of
+// a row in order (the last CTA to finish adds them).
+#include <algorithm>
+#include <cstring>
+
+#include "factor.h"
+#include "front.h"
+#include "internal.h"
+#include "prof.h"
+
+namespace hssnd {
+
+constexpr int MA_NT = 128, MA_ROWS = 128;
+template <class T> struct MultiTile {
+    static constexpr int KC = sizeof(T) == 4 ? 32 : 16;   // columns per chunk: 16 KB of the factor
+    static constexpr int VW = 16 / (int)sizeof(T);
+};
+
+template <class T> __device__ __forceinline__ void ldv(const T *p, T *a) {   // 16 bytes of shared memory
+    if constexpr (sizeof(T) == 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(p);
+        a[0] = v.x;
+        a[1] = v.y;
+        a[2] = v.z;
+        a[3] = v.w;
+    } else {
+        const double2 v = *reinterpret_cast<const double2 *>(p);
+        a[0] = v.x;
+        a[1] = v.y;
+    }
+}
+
+template <int BYTES> __device__ __forceinline__ void cp_async(void *dst, const void *src) {
+    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+
+// FWD: y = [F_ii^-1 P^t ; -F_bi F_ii^-1 P^t] x(Iperm)  ->  t = y[0,ni), x_B += y[ni,n)
+// BWD: x_I = t - W x_B
+template <class T, int RB, bool FWD>
+__global__ void __launch_bounds__(MA_NT) k_apply_multi(const ApplyItem *__restrict__ items,
+                                                     const FrontDev *__restrict__ fr, const T *__restrict__ arena,
+                                                     const int *__restrict__ iperm, const int *__restrict__ ilist,
+                                                     const int *__restrict__ blist,
+                                                     const ApplyParams *__restrict__ prm, T *__restrict__ part,
+                                                     int *__restrict__ tickets) {
+    pdl_launch_next();
+    constexpr int KC = MultiTile<T>::KC, VW = MultiTile<T>::VW;
+    constexpr int TR = RB == 32 ? 8 : 4, TC = RB == 8 ? 2 : 4;       // rows and vectors per thread
+    constexpr int RG = MA_ROWS / TR;                                  // row groups
+    constexpr int LDZ = RB + 16 / (int)sizeof(T);                     // vector block of a column, padded
+    __shared__ __align__(16) T As[2][KC][MA_ROWS];
+    __shared__ __align__(16) T Zs[2][KC][LDZ];
+    __shared__ int last_s;
+    const ApplyItem it = items[blockIdx.x];
+    const FrontDev F = fr[it.front];
+    const int tid = threadIdx.x;
+    const int nrows = FWD ? F.n : F.ni, colbase = FWD ? 0 : F.ni;
+    const T *M = arena + F.foff + it.row0 + (long)F.n * (colbase + it.c0);
+    const int ncol = it.c1 - it.c0, rows = min(MA_ROWS, nrows - it.row0);
+    const bool vec = F.n % VW == 0 && it.row0 % VW == 0;   // 16-byte columns (fronts start on 32 entries)
+    const int *list = FWD ? iperm + F.iperm_off + it.c0 : blist + F.bset_off + it.c0;
+    auto load_a = [&](int buf, int c0) {
+        if (vec) {
+            const bool full = rows == MA_ROWS;
+#pragma unroll
+            for (int q = 0; q < KC * MA_ROWS / VW / MA_NT; ++q) {
+                const int e = tid + MA_NT * q, c = e / (MA_ROWS / VW), r = (e % (MA_ROWS / VW)) * VW;
+                // (a piece past the last row stays inside the front's column or the next: rows % VW == 0)
+                if (c0 + c < ncol && (full || r < rows)) cp_async<16>(&As[buf][c][r], M + r + (long)F.n * (c0 + c));
+            }
+        } else {
+#pragma unroll 8
+            for (int q = 0; q < KC; ++q)
+                if (c0 + q < ncol && tid < rows) cp_async<(int)sizeof(T)>(&As[buf][q][tid], M + tid + (long)F.n * (c0 + q));
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    load_a(0, 0);
+    pdl_wait_prev();   // the vectors are the previous kernel's output
+    const double *w = prm->w;
+    const long ldw = prm->ldw;
+    const int nrhs = prm->nrhs;
+    constexpr int ZN = KC * RB / MA_NT;
+    T z[ZN];
+    auto load_z = [&](int c0) {
+#pragma unroll
+        for (int q = 0; q < ZN; ++q) {
+            const int e = tid + MA_NT * q, c = e % KC, r = e / KC;
+            z[q] = (c0 + c < ncol && r < nrhs) ? (T)w[list[c0 + c] + ldw * r] : T(0);
+        }
+    };
+    auto store_z = [&](int buf) {
+#pragma unroll
+        for (int q = 0; q < ZN; ++q) {
+            const int e = tid + MA_NT * q;
+            Zs[buf][e % KC][e / KC] = z[q];
+        }
+    };
+    // thread: rows r0(a) = 4 (tid % RG) + (a / 4) 64 + a % 4, vectors TC (tid / RG) ..
+    const int tr = tid % RG, tc = (tid / RG) * TC;
+    T acc[TR][TC];
+#pragma unroll
+    for (int a = 0; a < TR; ++a)
+#pragma unroll
+        for (int b = 0; b < TC; ++b) acc[a][b] = T(0);
+    load_z(0);
+    store_z(0);
+    for (int c0 = 0, buf = 0; c0 < ncol; c0 += KC, buf ^= 1) {
+        const bool more = c0 + KC < ncol;
+        if (more) {
+            load_a(buf ^ 1, c0 + KC);
+            load_z(c0 + KC);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const int kc = min(KC, ncol - c0);
+#pragma unroll 4
+        for (int q = 0; q < kc; ++q) {
+            T m[TR], x[TC];
+#pragma unroll
+            for (int a = 0; a < TR; a += VW) ldv(&As[buf][q][4 * tr + (a / 4) * 64 + a % 4], m + a);
+            if constexpr (TC >= VW) {
+#pragma unroll
+                for (int b = 0; b < TC; b += VW) ldv(&Zs[buf][q][tc + b], x + b);
+            } else {
+#pragma unroll
+                for (int b = 0; b < TC; ++b) x[b] = Zs[buf][q][tc + b];
+            }
+#pragma unroll
+            for (int a = 0; a < TR; ++a)
+#pragma unroll
+                for (int b = 0; b < TC; ++b) acc[a][b] = fma(m[a], x[b], acc[a][b]);
+        }
+        if (more) store_z(buf ^ 1);
+        __syncthreads();
+    }
+    auto row_of = [&](int a) { return 4 * tr + (a / 4) * 64 + a % 4; };
+    if (it.nchunk > 1) {
+        T *mine = part + (long)(it.first + it.chunk) * MA_ROWS * RB;
+#pragma unroll
+        for (int b = 0; b < TC; ++b)
+#pragma unroll
+            for (int a = 0; a < TR; ++a) mine[(tc + b) * MA_ROWS + row_of(a)] = acc[a][b];
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) last_s = atomicAdd(&tickets[it.tile], 1) == it.nchunk - 1;
+        __syncthreads();
+        if (!last_s) return;
+        __threadfence();
+        const T *p = part + (long)it.first * MA_ROWS * RB;
+#pragma unroll
+        for (int a = 0; a < TR; ++a)
+#pragma unroll
+            for (int b = 0; b < TC; ++b) acc[a][b] = T(0);
+        for (int ch = 0; ch < it.nchunk; ++ch, p += MA_ROWS * RB)
+#pragma unroll
+            for (int b = 0; b < TC; ++b)
+#pragma unroll
+                for (int a = 0; a < TR; ++a) acc[a][b] += __ldcg(p + (tc + b) * MA_ROWS + row_of(a));
+        if (tid == 0) tickets[it.tile] = 0;   // ready for the next apply
+    }
+    double *wv = prm->w, *tv = prm->tv;
+    const long ldt = prm->ldt;
+#pragma unroll
+    for (int a = 0; a < TR; ++a) {
+        const int i = it.row0 + row_of(a);
+        if (i >= nrows) continue;
+        const bool interior = !FWD || i < F.ni;
+        const int dof = interior ? ilist[F.iset_off + i] : blist[F.bset_off + i - F.ni];
+#pragma unroll
+        for (int b = 0; b < TC; ++b) {
+            const int r = tc + b;
+            if (r >= nrhs) continue;
+            const double y = (double)acc[a][b];
+            if (!FWD) wv[dof + ldw * r] = tv[dof + ldt * r] - y;
+            else if (interior) tv[dof + ldt * r] = y;
+            else wv[dof + ldw * r] += y;
+        }
+    }
+}
+
+// Columns per item of a front of order n: a split row tile writes and reads 128
+// x RB partial sums per item (16 KB in FP32 against 256 KB of the factor at 512
+// columns), and needs the split only where its level has few tiles.  By the
+// front alone, so that a forest sums as its instances do.
+static int multi_chunk(int n) { return n < 8192 ? 512 : 1024; }
+
+template <class T> int pack_apply_multi(hss_factor_t *F, cudaStream_t s) {
+    const size_t nst = F->apply.size();
+    std::vector<ApplyItem> items;
+    std::vector<ApplyMultiStage> &ms = F->multi;
+    ms.assign(nst, ApplyMultiStage{});
+    long part = 0;   // split items of a launch at most: the launches use one buffer in turn
+    int tk = 0;
+    for (size_t q = 0; q < nst; ++q) {
+        const ApplyStage &st = F->apply[q];
+        for (int pass = 0; pass < 2; ++pass) {
+            ms[q].off[pass] = (int)items.size();
+            ms[q].tk[pass] = tk;
+            int first = 0, tiles = 0;
+            for (int f = 0; f < (int)st.h_fronts.size(); ++f) {
+                const FrontDev &d = st.h_fronts[f];
+                if (d.ni == 0) continue;
+                const int nrows = pass == 0 ? d.n : d.ni, ncols = pass == 0 ? d.ni : d.nb;
+                const int chunk = multi_chunk(d.n), nch = std::max(1, cdiv(ncols, chunk));
+                for (int r0 = 0; r0 < nrows; r0 += MA_ROWS) {
+                    for (int ch = 0; ch < nch; ++ch) {
+                        ApplyItem it{f, r0, std::min(ncols, ch * chunk), std::min(ncols, (ch + 1) * chunk), -1, first, nch};
+                        it.chunk = ch;
+                        if (nch > 1) it.tile = tiles;
+                        items.push_back(it);
+                    }
+                    if (nch > 1) {
+                        first += nch;   // partial sums of split tiles only
+                        ++tiles;
+                    }
+                }
+            }
+            ms[q].cnt[pass] = (int)items.size() - ms[q].off[pass];
+            part = std::max(part, (long)first);
+            tk += tiles;
+        }
+    }
+    int rc;
+    if ((rc = F->multi_items.alloc(sizeof(ApplyItem) * std::max<size_t>(items.size(), 1))) ||
+        (rc = F->multi_tickets.alloc(sizeof(int) * std::max(tk, 1))))
+        return rc;
+    if ((rc = F->multi_part.alloc(sizeof(T) * MA_ROWS * APPLY_RB * std::max(part, 1L)))) return rc;
+    if (!items.empty())
+        HSS_CUDA(cudaMemcpyAsync(F->multi_items.p, items.data(), sizeof(ApplyItem) * items.size(), cudaMemcpyHostToDevice, s));
+    HSS_CUDA(cudaMemsetAsync(F->multi_tickets.p, 0, sizeof(int) * std::max(tk, 1), s));
+    // (a copy from pageable memory has left `items` by the time cudaMemcpyAsync returns)
+    return HSS_OK;
+}
+
+template <class T, int RB>
+cudaError_t launch_apply_multi(const hss_factor_t *F, size_t q, bool fwd, cudaStream_t s) {
+    const ApplyStage &st = F->apply[q];
+    const ApplyMultiStage &m = F->multi[q];
+    const int pass = fwd ? 0 : 1;
+    if (m.cnt[pass] == 0) return cudaSuccess;
+    const ApplyItem *items = F->multi_items.as<ApplyItem>() + m.off[pass];
+    T *part = F->multi_part.as<T>();
+    int *tk = F->multi_tickets.as<int>() + m.tk[pass];
+    const int *il = st.top ? F->d_topset.as<int>() : F->tree->d_iset.as<int>();
+    const int *bl = F->tree->d_bset.as<int>(), *ip = F->d_iperm.as<int>();
+    const FrontDev *fr = st.d_fronts;
+    const T *arena = F->arena_ptr<T>();
+    const ApplyParams *prm = F->d_aparams.as<ApplyParams>();
+    if (fwd)
+        return launch_pdl(k_apply_multi<T, RB, true>, dim3(m.cnt[pass]), dim3(MA_NT), 0, s, items, fr, arena, ip, il, bl,
+                          prm, part, tk);
+    return launch_pdl(k_apply_multi<T, RB, false>, dim3(m.cnt[pass]), dim3(MA_NT), 0, s, items, fr, arena, ip, il, bl,
+                      prm, part, tk);
+}
+
+#define INST(T)                                                                                            \
+    template int pack_apply_multi<T>(hss_factor_t *, cudaStream_t);                                         \
+    template cudaError_t launch_apply_multi<T, 8>(const hss_factor_t *, size_t, bool, cudaStream_t);        \
+    template cudaError_t launch_apply_multi<T, 16>(const hss_factor_t *, size_t, bool, cudaStream_t);       \
+    template cudaError_t launch_apply_multi<T, 32>(const hss_factor_t *, size_t, bool, cudaStream_t);
+INST(float)
+INST(double)
+#undef INST
+
+}  // namespace hssnd

@@ -22,6 +22,7 @@ namespace {
 constexpr int BK_NT = 256;
 constexpr int BK_CHUNK = 4096;
 constexpr int BK_MAXM = 32;   // largest restart length + 1
+constexpr int BK_NQ = 8;      // basis vectors per pass of the inner products
 
 struct BChunk {
     int p;          // process
@@ -42,24 +43,43 @@ __global__ void k_bdots(const double *__restrict__ V, long ldv, long vstride, in
     const BChunk C = ch[blockIdx.x];
     if (!act[C.p]) return;
     __shared__ double sh[BK_NT / 32][BK_MAXM + 1];
-    double acc[BK_MAXM];
-#pragma unroll
-    for (int q = 0; q < BK_MAXM; ++q) acc[q] = 0.0;
     const double *wc = w + (long)C.col * ldw + C.row0;
     const double *vc = V + (long)C.col * ldv + C.row0;
-    for (int i = threadIdx.x; i < C.len; i += BK_NT) {
-        const double wi = wc[i];
-#pragma unroll
-        for (int q = 0; q < BK_MAXM; ++q)
-            if (q < nq) acc[q] = fma(vc[i + vstride * q], wi, acc[q]);
-    }
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    // eight vectors at a time, four rows of each in flight per thread (w again
+    // from L1): 36 loads against one row's nq + 1 with all vectors at once,
+    // whose 32 accumulators left two CTAs per SM
+    for (int q0 = 0; q0 < nq; q0 += BK_NQ) {
+        double acc[BK_NQ];
 #pragma unroll
-    for (int q = 0; q < BK_MAXM; ++q) {
-        if (q >= nq) break;
-        double v = acc[q];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[wp][q] = v;
+        for (int q = 0; q < BK_NQ; ++q) acc[q] = 0.0;
+        const double *vq = vc + vstride * q0;
+        for (int i = threadIdx.x; i < C.len; i += 4 * BK_NT) {
+            double wi[4], v[BK_NQ][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) wi[u] = i + u * BK_NT < C.len ? wc[i + u * BK_NT] : 0.0;
+#pragma unroll
+            for (int q = 0; q < BK_NQ; ++q)
+                if (q0 + q < nq) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        v[q][u] = i + u * BK_NT < C.len ? vq[i + u * BK_NT + vstride * q] : 0.0;
+                }
+#pragma unroll
+            for (int q = 0; q < BK_NQ; ++q)
+                if (q0 + q < nq) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (i + u * BK_NT < C.len) acc[q] = fma(v[q][u], wi[u], acc[q]);
+                }
+        }
+#pragma unroll
+        for (int q = 0; q < BK_NQ; ++q) {
+            if (q0 + q >= nq) break;
+            double v = acc[q];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) sh[wp][q0 + q] = v;
+        }
     }
     __syncthreads();
     for (int q = threadIdx.x; q < nq; q += BK_NT) {

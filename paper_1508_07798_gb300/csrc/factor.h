@@ -20,6 +20,13 @@ struct ApplyItem {
     int tile;         // row-tile index inside the stage (ticket slot)
     int first;        // item index of the tile's first chunk
     int nchunk;       // chunks of this tile
+    int chunk;        // this item's place among them (several right-hand sides)
+};
+
+// Work items of a stage for several right-hand sides (apply_multi.cu), forward
+// and backward: their range in the factor's list and their tickets.
+struct ApplyMultiStage {
+    int off[2], cnt[2], tk[2];
 };
 
 // Per level (and the top block): fronts and the row tiles of the apply.
@@ -49,7 +56,10 @@ struct ApplyParams {
     int nrhs;
 };
 
-constexpr int APPLY_RB = 8;   // right-hand sides per sweep of the multi-RHS apply (factor read once per 8)
+// Right-hand sides per sweep of the apply: 1, or blocks of up to 8, 16 or 32
+// (the factor is read once per sweep).
+constexpr int APPLY_RB = 32;
+constexpr int APPLY_SLOTS = 4;
 
 struct FrontLog {   // per-front record (rank logging, Sec. 5 empirical cost)
     int box, level, ni, nb, r, rounds, kmax, nnodes;
@@ -63,6 +73,10 @@ int pack_apply(hss_factor_t *F, cudaStream_t s);
 // Chooses each stage's forward and backward column chunk by timing the
 // candidates (process-wide cache keyed by the stage's front shapes).
 int tune_apply(hss_factor_t *F, cudaStream_t s);
+// Several right-hand sides: the work items (at a factor's first such apply) and
+// the launch of one stage and direction.
+template <class T> int pack_apply_multi(hss_factor_t *F, cudaStream_t s);
+template <class T, int RB> cudaError_t launch_apply_multi(const hss_factor_t *F, size_t stage, bool fwd, cudaStream_t s);
 int ilu_apply(const hss_ilu_t *M, int nrhs, const double *x, long ldx, double *y, long ldy, cudaStream_t s);
 long ilu_ndof(const hss_ilu_t *M);
 int spmv(const hss_bsr *A, int nrhs, const double *x, long ldx, double *y, long ldy, cudaStream_t s);
@@ -109,11 +123,13 @@ struct hss_factor_t {
     double host_sync_ms = 0;   // host time spent waiting in them
     double host_ms = 0;        // host time of the whole call
     double host_gap_ms = 0;    // host time from each read-back to the next kernel launch (device idle)
-    // captured apply sweeps (slot 0: one right-hand side, slot 1: blocks of APPLY_RB)
-    cudaGraphExec_t gexec[2] = {nullptr, nullptr};
-    int graph_kernels[2] = {0, 0};
+    // captured apply sweeps (slot 0: one right-hand side, 1..3: blocks of 8, 16, 32)
+    cudaGraphExec_t gexec[hssnd::APPLY_SLOTS] = {};
+    int graph_kernels[hssnd::APPLY_SLOTS] = {};
+    std::vector<hssnd::ApplyMultiStage> multi;   // per stage, filled by the first apply to several vectors
+    hssnd::DevBuf multi_items, multi_tickets, multi_part;
     hssnd::DevBuf d_aparams;
-    hssnd::DevBuf d_apart;       // partial sums of split apply tiles (items x 32 x 4)
+    hssnd::DevBuf d_apart;       // partial sums of split apply tiles (items x 32)
     hssnd::DevBuf d_tickets;     // one ticket counter per split tile
     hssnd::DevBuf apply_buf;     // fronts and work items of every apply stage, one allocation
     // subtree part of the apply: stages [0, sub_nst) (the deepest levels) run
