@@ -9,8 +9,12 @@
 // value once per 128 rows.  The kernel for one vector broadcasts x by shuffles,
 // one per product: with 8 vectors it was bound by the shuffle rate, a quarter
 // of the FMA rate, read the factor again for every 8 and gathered x for every
-// 32 rows.  Sums run over the columns of an item in order and over the items of
-// a row in order (the last CTA to finish adds them).
+// 32 rows.  Sums run over segments of `seg` columns, then over the segments and
+// the items of a row in order (the last CTA to finish adds the items): up to 512
+// columns the order of the kernel for one vector, whose work items the segments are.
+// 20 vectors, 32^3 diffusion (8.5 GB): 12.6 -> 5.0 ms per apply; 32 vectors, 24
+// instances of 16..64^2, p = 2: 5.5 -> 2.4 ms; bound by the shared-memory loads
+// of the products (three of 16 bytes per 32 FMAs).
 #include <algorithm>
 #include <cstring>
 
@@ -57,7 +61,7 @@ __global__ void __launch_bounds__(MA_NT) k_apply_multi(const ApplyItem *__restri
                                                      const int *__restrict__ iperm, const int *__restrict__ ilist,
                                                      const int *__restrict__ blist,
                                                      const ApplyParams *__restrict__ prm, T *__restrict__ part,
-                                                     int *__restrict__ tickets) {
+                                                     int *__restrict__ tickets, int seg) {
     pdl_launch_next();
     constexpr int KC = MultiTile<T>::KC, VW = MultiTile<T>::VW;
     constexpr int TR = RB == 32 ? 8 : 4, TC = RB == 8 ? 2 : 4;       // rows and vectors per thread
@@ -113,11 +117,11 @@ __global__ void __launch_bounds__(MA_NT) k_apply_multi(const ApplyItem *__restri
     };
     // thread: rows r0(a) = 4 (tid % RG) + (a / 4) 64 + a % 4, vectors TC (tid / RG) ..
     const int tr = tid % RG, tc = (tid / RG) * TC;
-    T acc[TR][TC];
+    T acc[TR][TC], sum[TR][TC];   // of the segment, of the segments before it
 #pragma unroll
     for (int a = 0; a < TR; ++a)
 #pragma unroll
-        for (int b = 0; b < TC; ++b) acc[a][b] = T(0);
+        for (int b = 0; b < TC; ++b) acc[a][b] = sum[a][b] = T(0);
     load_z(0);
     store_z(0);
     for (int c0 = 0, buf = 0; c0 < ncol; c0 += KC, buf ^= 1) {
@@ -149,6 +153,15 @@ __global__ void __launch_bounds__(MA_NT) k_apply_multi(const ApplyItem *__restri
                 for (int b = 0; b < TC; ++b) acc[a][b] = fma(m[a], x[b], acc[a][b]);
         }
         if (more) store_z(buf ^ 1);
+        if (!more || (c0 + KC) % seg == 0) {
+#pragma unroll
+            for (int a = 0; a < TR; ++a)
+#pragma unroll
+                for (int b = 0; b < TC; ++b) {
+                    sum[a][b] += acc[a][b];
+                    acc[a][b] = T(0);
+                }
+        }
         __syncthreads();
     }
     auto row_of = [&](int a) { return 4 * tr + (a / 4) * 64 + a % 4; };
@@ -157,7 +170,7 @@ __global__ void __launch_bounds__(MA_NT) k_apply_multi(const ApplyItem *__restri
 #pragma unroll
         for (int b = 0; b < TC; ++b)
 #pragma unroll
-            for (int a = 0; a < TR; ++a) mine[(tc + b) * MA_ROWS + row_of(a)] = acc[a][b];
+            for (int a = 0; a < TR; ++a) mine[(tc + b) * MA_ROWS + row_of(a)] = sum[a][b];
         __threadfence();
         __syncthreads();
         if (tid == 0) last_s = atomicAdd(&tickets[it.tile], 1) == it.nchunk - 1;
@@ -168,12 +181,12 @@ __global__ void __launch_bounds__(MA_NT) k_apply_multi(const ApplyItem *__restri
 #pragma unroll
         for (int a = 0; a < TR; ++a)
 #pragma unroll
-            for (int b = 0; b < TC; ++b) acc[a][b] = T(0);
+            for (int b = 0; b < TC; ++b) sum[a][b] = T(0);
         for (int ch = 0; ch < it.nchunk; ++ch, p += MA_ROWS * RB)
 #pragma unroll
             for (int b = 0; b < TC; ++b)
 #pragma unroll
-                for (int a = 0; a < TR; ++a) acc[a][b] += __ldcg(p + (tc + b) * MA_ROWS + row_of(a));
+                for (int a = 0; a < TR; ++a) sum[a][b] += __ldcg(p + (tc + b) * MA_ROWS + row_of(a));
         if (tid == 0) tickets[it.tile] = 0;   // ready for the next apply
     }
     double *wv = prm->w, *tv = prm->tv;
@@ -188,7 +201,7 @@ __global__ void __launch_bounds__(MA_NT) k_apply_multi(const ApplyItem *__restri
         for (int b = 0; b < TC; ++b) {
             const int r = tc + b;
             if (r >= nrhs) continue;
-            const double y = (double)acc[a][b];
+            const double y = (double)sum[a][b];
             if (!FWD) wv[dof + ldw * r] = tv[dof + ldt * r] - y;
             else if (interior) tv[dof + ldt * r] = y;
             else wv[dof + ldw * r] += y;
@@ -264,11 +277,12 @@ cudaError_t launch_apply_multi(const hss_factor_t *F, size_t q, bool fwd, cudaSt
     const FrontDev *fr = st.d_fronts;
     const T *arena = F->arena_ptr<T>();
     const ApplyParams *prm = F->d_aparams.as<ApplyParams>();
+    const int seg = (int)q < F->sub_nst ? 1 << 30 : st.chunk[pass];   // (a subtree's item holds every column)
     if (fwd)
         return launch_pdl(k_apply_multi<T, RB, true>, dim3(m.cnt[pass]), dim3(MA_NT), 0, s, items, fr, arena, ip, il, bl,
-                          prm, part, tk);
+                          prm, part, tk, seg);
     return launch_pdl(k_apply_multi<T, RB, false>, dim3(m.cnt[pass]), dim3(MA_NT), 0, s, items, fr, arena, ip, il, bl,
-                      prm, part, tk);
+                      prm, part, tk, seg);
 }
 
 #define INST(T)                                                                                            \
