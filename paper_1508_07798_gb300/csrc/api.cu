@@ -20,26 +20,61 @@ void count_alloc() { g_alloc_requests.fetch_add(1, std::memory_order_relaxed); }
 
 void set_error(const std::string &msg) { g_last_error = msg; }
 
+static void scratch_cache_trim();
+
 int cuda_fail(cudaError_t e, const char *what) {
     g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
     if (e == cudaErrorMemoryAllocation) return HSS_ENOMEM;
     return HSS_ECUDA;
 }
 
-int DevBuf::alloc(size_t nbytes) {
-    if (nbytes <= bytes && p) return HSS_OK;
-    release();
-    if (nbytes == 0) nbytes = 1;
-    count_alloc();
-    cudaError_t e = cudaMalloc(&p, nbytes);
+// cudaMalloc, with the cached memory given back first when it fails
+static int raw_alloc(DevBuf &b, size_t nbytes) {
+    cudaError_t e = cudaMalloc(&b.p, nbytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        scratch_cache_trim();
+        e = cudaMalloc(&b.p, nbytes);
+    }
     if (e != cudaSuccess) {
-        p = nullptr;
+        b.p = nullptr;
         cudaGetLastError();
         set_error("cudaMalloc of " + std::to_string(nbytes) + " bytes failed: " + cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? HSS_ENOMEM : HSS_ECUDA;
     }
-    bytes = nbytes;
+    b.bytes = nbytes;
+    if (cudaGetDevice(&b.dev) != cudaSuccess) b.dev = 0;
     return HSS_OK;
+}
+
+int DevBuf::alloc(size_t nbytes) {
+    if (nbytes <= bytes && p) return HSS_OK;
+    release();
+    if (nbytes == 0) nbytes = 1;
+    // sizes in steps of an eighth of their power of two (exact from 1 GB), so
+    // that a slightly different structure finds the memory of the last one
+    size_t want = nbytes;
+    if (nbytes < ((size_t)1 << 30)) {
+        size_t step = 512;
+        while (step * 16 <= nbytes) step *= 2;
+        want = (nbytes + step - 1) / step * step;
+    }
+    return scratch_cache_take_device(nbytes, want, *this);
+}
+
+void DevBuf::release() {
+    if (!p) return;
+    int cur = 0;
+    const bool other = cudaGetDevice(&cur) == cudaSuccess && cur != dev;
+    if (other) cudaSetDevice(dev);
+    if (cudaDeviceSynchronize() == cudaSuccess) {
+        scratch_cache_give_device(std::move(*this));
+    } else {   // (a failed device, or a capture in progress: leave it to the driver)
+        cudaGetLastError();
+        cudaFree(p);
+        forget();
+    }
+    if (other) cudaSetDevice(cur);
 }
 
 // Dynamic shared-memory limit of a kernel, set once per (device, kernel):
@@ -93,36 +128,59 @@ int current_device() {
 }
 }  // namespace
 
+// A cached chunk of at least want bytes, else of at least min; not one so much
+// larger that a later, larger request would miss it; else fresh memory.
 int scratch_cache_take_device(size_t min_bytes, size_t want_bytes, DevBuf &out) {
     count_alloc();
     const int d = current_device();
+    const size_t most = std::max(4 * want_bytes, (size_t)64 << 10);
     {
         std::lock_guard<std::mutex> lk(cache().mu);
         auto &v = cache().dev;
-        int best = -1;
-        for (int k = 0; k < (int)v.size(); ++k)
-            if (v[k].first == d && v[k].second.bytes >= min_bytes &&
-                (best < 0 || v[k].second.bytes < v[best].second.bytes))
-                best = k;
-        if (best >= 0) {
-            out = std::move(v[best].second);
-            cache().dev_bytes -= out.bytes;
-            v.erase(v.begin() + best);
-            return HSS_OK;
+        for (size_t least : {want_bytes, min_bytes}) {
+            int best = -1;
+            for (int k = 0; k < (int)v.size(); ++k)
+                if (v[k].first == d && v[k].second.bytes >= least && v[k].second.bytes <= most &&
+                    (best < 0 || v[k].second.bytes < v[best].second.bytes))
+                    best = k;
+            if (best >= 0) {
+                out = std::move(v[best].second);
+                cache().dev_bytes -= out.bytes;
+                v.erase(v.begin() + best);
+                return HSS_OK;
+            }
         }
     }
-    return out.alloc(want_bytes);
+    return raw_alloc(out, want_bytes);
 }
 
+// Nothing queued on the device may still use b (its caller has waited).
 void scratch_cache_give_device(DevBuf &&b) {
     if (!b.p) return;
-    std::lock_guard<std::mutex> lk(cache().mu);
-    if (cache().dev_bytes + b.bytes > CACHE_DEV_MAX) {
-        b.release();
-        return;
+    {
+        std::lock_guard<std::mutex> lk(cache().mu);
+        if (cache().dev_bytes + b.bytes <= CACHE_DEV_MAX) {
+            cache().dev_bytes += b.bytes;
+            const int d = b.dev;
+            cache().dev.emplace_back(d, std::move(b));
+            return;
+        }
     }
-    cache().dev_bytes += b.bytes;
-    cache().dev.emplace_back(current_device(), std::move(b));
+    cudaFree(b.p);
+    b.forget();
+}
+
+static void scratch_cache_trim() {
+    std::vector<std::pair<int, DevBuf>> v;
+    {
+        std::lock_guard<std::mutex> lk(cache().mu);
+        v.swap(cache().dev);
+        cache().dev_bytes = 0;
+    }
+    for (auto &c : v) {
+        cudaFree(c.second.p);
+        c.second.forget();
+    }
 }
 
 void *scratch_cache_take_pinned(size_t min_bytes, size_t want_bytes, size_t &got) {

@@ -63,33 +63,35 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
         if (_e != cudaSuccess) return cuda_fail(_e, "shared-memory attribute of " #kernel); \
     } while (0)
 
-// Device allocation owned by a handle.
+// Device allocation owned by a handle or a call.  Memory comes from the
+// process-wide cache below and goes back to it when the buffer is released,
+// after the device has finished what was launched (the wait that cudaFree
+// implies), so the handles of a program that factors again and again cost no
+// cudaMalloc and cudaFree.
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    int dev = 0;
     DevBuf() = default;
     DevBuf(const DevBuf &) = delete;
     DevBuf &operator=(const DevBuf &) = delete;
-    DevBuf(DevBuf &&o) noexcept : p(o.p), bytes(o.bytes) {
-        o.p = nullptr;
-        o.bytes = 0;
-    }
+    DevBuf(DevBuf &&o) noexcept : p(o.p), bytes(o.bytes), dev(o.dev) { o.forget(); }
     DevBuf &operator=(DevBuf &&o) noexcept {
         if (this != &o) {
             release();
             p = o.p;
             bytes = o.bytes;
-            o.p = nullptr;
-            o.bytes = 0;
+            dev = o.dev;
+            o.forget();
         }
         return *this;
     }
     ~DevBuf() { release(); }
-    void release() {
-        if (p) cudaFree(p);
+    void forget() {
         p = nullptr;
         bytes = 0;
     }
+    void release();
     int alloc(size_t nbytes);  // returns HSS_OK / HSS_ENOMEM
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
@@ -151,7 +153,9 @@ struct ScratchPtr {
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
 
-// Process-wide cache of scratch memory (bounded; thread-safe).
+// Process-wide cache of device and pinned memory: thread-safe, at most 8 GB of
+// device memory and 512 MB pinned; a device allocation that fails gives the
+// cached memory back to the driver and tries again.
 int scratch_cache_take_device(size_t min_bytes, size_t want_bytes, DevBuf &out);
 void scratch_cache_give_device(DevBuf &&b);
 void *scratch_cache_take_pinned(size_t min_bytes, size_t want_bytes, size_t &got);
