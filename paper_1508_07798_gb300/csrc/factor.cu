@@ -138,7 +138,8 @@ static uint64_t shape_key(const GemmDesc<float> &d, int tc_kind) {
 static int time_engine(const Engine &E, const GemmDesc<float> &d, int eng, Work &W, cudaStream_t s, float *ms) {
     std::vector<GemmDesc<float>> dv{d};
     std::vector<GemmTile> tl;
-    if (eng == ENG_SIMT) gemm_tiles_for(d, 0, tl);
+    const int ts = gemm_tile_size<float>({&d});
+    if (eng == ENG_SIMT) gemm_tiles_for(d, 0, tl, ts);
     else gemm_tc_tiles_for(d, 0, tl);
     GemmDesc<float> *dd;
     GemmTile *dt;
@@ -147,7 +148,7 @@ static int time_engine(const Engine &E, const GemmDesc<float> &d, int eng, Work 
     if ((rc = W.up(dv, &dd)) || (rc = W.up(tl, &dt))) return rc;
     if (eng == ENG_TMA && (rc = gemm_tma_descs(dv, std::vector<char>{1}, W, &td))) return rc;
     auto launch = [&]() -> int {
-        if (eng == ENG_SIMT) return gemm_batched<float>(dd, dt, (int)tl.size(), s, 0.0);
+        if (eng == ENG_SIMT) return gemm_batched<float>(dd, dt, (int)tl.size(), s, 0.0, ts);
         if (eng == ENG_TMA) return gemm_tma(td, dt, (int)tl.size(), E.err, s, 0.0);
         return gemm_tc(dd, dt, (int)tl.size(), E.tc == 2 ? 0 : 1, E.err, s, 0.0);
     };
@@ -239,6 +240,7 @@ template <class T> struct GemmPlan {
     std::vector<GemmTile> tl[NENG];
     std::vector<int> off[NENG];
     std::vector<double> fl[NENG];
+    std::vector<int> ts;         // tile size of each group's SIMT launch
     TmaGemmDesc *d_tdescs = nullptr;
     GemmTile *d_tl[NENG] = {};
     // ENG_H2: tiles refer to h2 (the flagged problems only), images shared by the groups
@@ -284,7 +286,12 @@ int plan_gemms(const Engine &E, const std::vector<GemmDesc<T>> &descs, const std
         }
         if (most && (rc = W.dalloc(most, &h2_ws))) return rc;
     }
+    P.ts.assign(ngroups, GEMM_TM);
     for (int g = 0; g < ngroups; ++g) {
+        std::vector<const GemmDesc<T> *> simt;
+        for (int i : of[g])
+            if (which[i] == ENG_SIMT) simt.push_back(&descs[i]);
+        P.ts[g] = gemm_tile_size<T>(simt);
         for (int e = 0; e < NENG; ++e) P.off[e][g] = (int)P.tl[e].size();
         P.split_off[g] = (int)P.split.size();
         size_t h2_off = 0;
@@ -299,7 +306,7 @@ int plan_gemms(const Engine &E, const std::vector<GemmDesc<T>> &descs, const std
                     continue;
                 }
             }
-            if (e == ENG_SIMT) gemm_tiles_for(descs[i], i, P.tl[e]);
+            if (e == ENG_SIMT) gemm_tiles_for(descs[i], i, P.tl[e], P.ts[g]);
             else if constexpr (std::is_same<T, float>::value) gemm_tc_tiles_for(descs[i], i, P.tl[e]);
             P.fl[e][g] += gemm_flops(descs[i]);
         }
@@ -330,7 +337,7 @@ int run_gemm_group(const Engine &E, const GemmPlan<T> &P, const GemmDesc<T> *d_d
         if (n <= 0) continue;
         const GemmTile *t = P.d_tl[e] + P.off[e][g];
         if (e == ENG_SIMT) {
-            rc = gemm_batched<T>(d_descs, t, n, s, P.fl[e][g]);
+            rc = gemm_batched<T>(d_descs, t, n, s, P.fl[e][g], P.ts[g]);
         } else if constexpr (std::is_same<T, float>::value) {
             if ((e == ENG_TMA || e == ENG_BF16) && !P.d_tdescs) {
                 set_error("GEMM plan: tensor-core tiles without tensor maps");
@@ -744,6 +751,23 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
             return rc;
         HSS_CUDA(cudaMemsetAsync(d_kout, 0, sizeof(int) * 2 * nn, s));
         HSS_CUDA(cudaMemsetAsync(d_fk, 0, sizeof(int) * nc, s));
+        // ---- the test matrices' sign bits (Omega, Psi per front)
+        std::vector<SignBlock> sblk;
+        std::vector<long> soff(2 * nc);   // of (front, stream)
+        long swords = 0;
+        for (int c = 0; c < nc; ++c)
+            for (int strm = 0; strm < 2; ++strm) {
+                const int ldw = cdiv(cfs[c].r, 32), words = cfs[c].nb * ldw;
+                soff[2 * c + strm] = swords;
+                for (int w0 = 0; w0 < words; w0 += SIGN_WORDS)
+                    sblk.push_back({swords, ldw, strm, cfs[c].box, w0, std::min(SIGN_WORDS, words - w0)});
+                swords += words;
+            }
+        SignBlock *d_sblk;
+        uint32_t *d_bits;
+        if ((rc = W.up(sblk, &d_sblk)) || (rc = W.dalloc((size_t)swords, &d_bits)) ||
+            (rc = launch_sign_bits(d_sblk, (int)sblk.size(), o.seed, d_bits, s)))
+            return rc;
         // ---- sampling Y = S Omega, Z = S^t Psi, then the leaf corrections
         std::vector<GemmDesc<T>> g1, g2;
         std::vector<GemmTile> t2;   // leaf corrections (SIMT)
@@ -763,13 +787,16 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
             d.front = cfs[c].box;
             d.brow0 = 0;
             d.ldc = cfs[c].nb;
+            d.ldw = cdiv(cfs[c].r, 32);
             d.C = ws + cfs[c].yoff;
             d.transA = 0;
             d.stream = 0;
+            d.bits = d_bits + soff[2 * c];
             g1.push_back(d);
             d.C = ws + cfs[c].zoff;
             d.transA = 1;
             d.stream = 1;
+            d.bits = d_bits + soff[2 * c + 1];
             g1.push_back(d);
             for (int i = node_base[c]; i < node_base[c + 1]; ++i) {
                 if (nodes[i].a >= 0) continue;
@@ -784,13 +811,13 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
                 e.C = ws + cfs[c].yoff + lo;
                 e.transA = 0;
                 e.stream = 0;
+                e.bits = d_bits + soff[2 * c];
                 g2.push_back(e);
-                gemm_tiles_for(g2.back(), (int)g2.size() - 1, t2);
                 e.C = ws + cfs[c].zoff + lo;
                 e.transA = 1;
                 e.stream = 1;
+                e.bits = d_bits + soff[2 * c + 1];
                 g2.push_back(e);
-                gemm_tiles_for(g2.back(), (int)g2.size() - 1, t2);
             }
         }
         {
@@ -798,13 +825,17 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
             GemmDesc<T> *a, *c2;
             GemmTile *d2;
             GemmPlan<T> plan;
+            std::vector<const GemmDesc<T> *> all2;
+            for (const auto &d : g2) all2.push_back(&d);
+            const int ts2 = gemm_tile_size<T>(all2);
+            for (size_t i = 0; i < g2.size(); ++i) gemm_tiles_for(g2[i], (int)i, t2, ts2);
             if ((rc = W.up(g1, &a)) || (rc = W.up(g2, &c2)) || (rc = W.up(t2, &d2)) ||
                 (rc = plan_gemms<T>(eng, g1, std::vector<int>(g1.size(), 0), 1, plan, W, s)))
                 return rc;
             double f2 = 0;
             for (auto &d : g2) f2 += gemm_flops(d);
             if ((rc = run_gemm_group<T>(eng, plan, a, 0, s, "gemm_tma_sample"))) return rc;
-            if ((rc = gemm_batched<T>(c2, d2, (int)t2.size(), s, f2))) return rc;
+            if ((rc = gemm_batched<T>(c2, d2, (int)t2.size(), s, f2, ts2))) return rc;
         }
         // ---- interpolative decompositions, deepest HSS level first
         HSS_HOST("compress_id_decide_expand");

@@ -204,7 +204,9 @@ namespace hssnd {
 // ---------------------------------------------------------------- gemm
 // C = alpha * op(A) * op(B) + beta * C on a list of column-major problems.
 // B == nullptr: op(B)(kk, j) is the +-1 test matrix entry of (seed, stream,
-// front, row brow0 + kk, column j) (counter-based SplitMix64 sign).
+// front, row brow0 + kk, column j) (counter-based SplitMix64 sign), which the
+// SIMT kernel reads as sign bits: word j / 32 of row brow0 + kk at ldw words a
+// row (1: -1).
 // Rows [zr_lo, zr_hi) use beta = 0; columns [skip_lo, skip_hi) are not written.
 template <class T> struct GemmDesc {
     const T *A;
@@ -218,7 +220,17 @@ template <class T> struct GemmDesc {
     int skip_lo, skip_hi;
     uint64_t seed;
     int stream, front, brow0;
+    const uint32_t *bits;
+    int ldw;
 };
+
+// Words [word0, word0 + words) of a test matrix's sign bits: rows of ldw words
+// from word off on (k_sign_bits).
+struct SignBlock {
+    long off;
+    int ldw, stream, front, word0, words;
+};
+constexpr int SIGN_WORDS = 256;   // words of a block at most
 
 struct GemmTile {
     int desc;
@@ -230,9 +242,17 @@ constexpr int GEMM_TN = 64;
 constexpr int GEMM_TC_TM = 128;   // tile of the tcgen05 GEMM (one MMA M x N)
 constexpr int GEMM_TC_TN = 128;
 
+// ts: the tile size (64 or 32) the list was made for
 template <class T>
 int gemm_batched(const GemmDesc<T> *d_desc, const GemmTile *d_tiles, int ntiles, cudaStream_t s,
-                 double flops = 0.0);
+                 double flops = 0.0, int ts = GEMM_TM);
+// Tile size of a launch of these problems: 32 below so many 64 x 64 tiles (about
+// one and a half waves of them: launches of 36 to 1,000 tiles are most of a
+// factorization's; limits of 600 and 2,000 measured alike, always 64 cost the 64 x
+// 64, p = 2 factorization 0.8 ms, always 32 the p = 3 one 0.4 ms).
+template <class T> int gemm_tile_size(const std::vector<const GemmDesc<T> *> &group);
+constexpr long GEMM_SMALL_LIMIT = 2000;
+int launch_sign_bits(const SignBlock *d_blocks, int nblocks, uint64_t seed, uint32_t *out, cudaStream_t s);
 
 // Tensor-core (tcgen05, TF32) GEMM of the FP32 form: split = 1 uses the
 // three-product hi/lo split (FP32 accuracy), 0 a single TF32 product.  err is
@@ -271,7 +291,7 @@ template <class T> double gemm_flops(const GemmDesc<T> &d) {
 }
 
 template <class T>
-void gemm_tiles_for(const GemmDesc<T> &d, int desc_index, std::vector<GemmTile> &tiles);
+void gemm_tiles_for(const GemmDesc<T> &d, int desc_index, std::vector<GemmTile> &tiles, int ts = GEMM_TM);
 
 // ---------------------------------------------------------------- device helpers
 __host__ __device__ inline uint64_t splitmix64(uint64_t x) {
