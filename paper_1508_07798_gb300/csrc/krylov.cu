@@ -2,9 +2,10 @@
 //
 // The paper measures its preconditioner by GMRES iterations (Sec. 5).  Each
 // Arnoldi step here: z_j = M^-1 v_j (hss_apply), w = A z_j (SpMV), classical
-// Gram-Schmidt applied twice against V (two reductions + updates each), the
-// new basis vector, and one Givens rotation of the Hessenberg column, all on
-// the device.  The host reads one residual estimate per step to stop.
+// Gram-Schmidt applied twice against V, the new basis vector, and one Givens
+// rotation of the Hessenberg column, in four launches on the device.  The host
+// reads one residual estimate per step to stop.
+#include <algorithm>
 #include <cmath>
 
 #include "factor.h"
@@ -14,7 +15,7 @@ namespace hssnd {
 
 constexpr int KRY_NT = 256;
 constexpr int KRY_MAXM = 32;      // largest restart length + 1
-constexpr int DOT_BLOCKS = 304;   // 2 x 152 SMs
+constexpr int DOT_BLOCKS = 304;   // blocks of rows: 2 per SM
 
 // y = A x, one thread per scalar row and right-hand side (any block size).
 __global__ void k_spmv(int nb, int bs, const int *__restrict__ row_ptr, const int *__restrict__ col_idx,
@@ -135,145 +136,247 @@ __global__ void k_spmv_multi(int nb, int bs, const int *__restrict__ row_ptr, co
     }
 }
 
-// partial[b * KRY_MAXM + q] = sum over this CTA's rows of V(:,q) . w, q < nq
-__global__ void k_dots(const double *__restrict__ V, long ldv, int nq, const double *__restrict__ w, long N,
-                       double *__restrict__ partial) {
+// The vector kernels of a GMRES step.  Rows are dealt to DOT_BLOCKS blocks of
+// KRY_NT; CTA c holds blocks c and c + GS_GRID, so few rows spread over all SMs
+// and every SM adds up the partial sums once.  An inner product leaves one
+// partial per block in part[q * DOT_BLOCKS + block]; the kernel that needs the
+// sum adds the partials in every CTA, in one fixed order, instead of a launch of
+// its own.  What bounds them is launches and the FP64 pipe (a warp's DFMA takes
+// 64 clocks of its scheduler), not the vectors, which are in L2: 64 x 64 quads,
+// p = 2 (36,864 dofs), one Arnoldi step of the first five: 13 launches, 100 us when
+// timed one by one -> 4 launches, 23 us; the solve 1,185 -> 1,016 us.
+constexpr int GS_GRID = DOT_BLOCKS / 2, GS_NT = 2 * KRY_NT, GS_NW = GS_NT / 32;
+
+static int gs_grid(long N) { return (int)std::max(1L, std::min((long)GS_GRID, (N + KRY_NT - 1) / KRY_NT)); }
+
+// a[q] summed over the block's threads into part, q < nq.  The lanes of a warp
+// halve the list of q's at each exchange (NQ - 1 additions a lane instead of
+// 5 NQ; the additions are the tree of a shuffle-down, so the sum is the same).
+template <int NQ>
+__device__ __forceinline__ void block_partials(double (&a)[NQ], int nq, long N, double *__restrict__ part) {
+    __shared__ double sh[GS_NW][NQ];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int LQ = NQ == 1 ? 0 : NQ == 2 ? 1 : NQ == 4 ? 2 : NQ == 8 ? 3 : NQ == 16 ? 4 : 5;
+    const int half = threadIdx.x / KRY_NT, blk = blockIdx.x + GS_GRID * half;
+    if ((long)blk * KRY_NT < N) {   // uniform over the half's warps
+#pragma unroll
+        for (int t = 0; t < 5; ++t) {
+            const int o = 16 >> t;
+            if (t < LQ) {
+                const int n = NQ >> (t + 1);
+                const bool up = lane & o;
+#pragma unroll
+                for (int k = 0; k < n; ++k) {
+                    const double send = up ? a[k] : a[k + n], keep = up ? a[k + n] : a[k];
+                    a[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            } else
+                a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+        }
+        if ((lane & ((32 >> LQ) - 1)) == 0) sh[w][lane >> (5 - LQ)] = a[0];
+    }
+    __syncthreads();
+    const int q = threadIdx.x % KRY_NT;
+    if (q < nq && (long)blk * KRY_NT < N) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < KRY_NT / 32; ++k) s += sh[half * (KRY_NT / 32) + k][q];
+        part[q * DOT_BLOCKS + blk] = s;
+    }
+}
+
+// hs[q] = the partials' sum, q < nq: one warp per q, fixed order.
+__device__ __forceinline__ void sum_partials(const double *__restrict__ part, int nq, long N, double *hs) {
+    const int lane = threadIdx.x & 31;
+    const int nblk = (int)std::min((long)DOT_BLOCKS, (N + KRY_NT - 1) / KRY_NT);   // blocks that hold rows
+    for (int q = threadIdx.x >> 5; q < nq; q += GS_NW) {
+        constexpr int PER = (DOT_BLOCKS + 31) / 32;
+        double v[PER], s = 0.0;
+#pragma unroll
+        for (int t = 0; t < PER; ++t) v[t] = lane + 32 * t < nblk ? __ldcg(part + q * DOT_BLOCKS + lane + 32 * t) : 0.0;
+#pragma unroll
+        for (int t = 0; t < PER; ++t)
+            if (32 * t < nblk) s += v[t];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) hs[q] = s;
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ long gs_row() {
+    return (long)(blockIdx.x + GS_GRID * (threadIdx.x / KRY_NT)) * KRY_NT + threadIdx.x % KRY_NT;
+}
+
+// partials of V(:, q) . w, q < nq <= NQ
+template <int NQ>
+__global__ void __launch_bounds__(GS_NT) k_gs_dots(const double *__restrict__ V, long ldv, int nq,
+                                                 const double *__restrict__ w, long N, double *__restrict__ part) {
     pdl_launch_next();
     pdl_wait_prev();
-    __shared__ double sh[KRY_NT / 32][KRY_MAXM + 1];
-    double acc[KRY_MAXM];
+    double acc[NQ];
 #pragma unroll
-    for (int q = 0; q < KRY_MAXM; ++q) acc[q] = 0.0;
-    for (long i = (long)blockIdx.x * KRY_NT + threadIdx.x; i < N; i += (long)gridDim.x * KRY_NT) {
-        double wi = w[i];
+    for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
+    for (long i = gs_row(); i < N; i += DOT_BLOCKS * KRY_NT) {
+        const double wi = w[i];
 #pragma unroll
-        for (int q = 0; q < KRY_MAXM; ++q)
+        for (int q = 0; q < NQ; ++q)
             if (q < nq) acc[q] = fma(V[i + ldv * q], wi, acc[q]);
     }
-    int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    block_partials<NQ>(acc, nq, N, part);
+}
+
+// One pass of classical Gram-Schmidt: h = the sums of part, w -= V(:, 0:nq) h, and
+//   first pass:  partials of V(:, q) . w to part2;  hcol = h
+//   second pass: partial of w . w to part2;         hcol += h
+template <int NQ, bool SECOND>
+__global__ void __launch_bounds__(GS_NT) k_gs_sub(const double *__restrict__ V, long ldv, int nq,
+                                                double *__restrict__ w, long N, const double *__restrict__ part,
+                                                double *__restrict__ part2, double *__restrict__ hcol) {
+    pdl_launch_next();
+    pdl_wait_prev();
+    __shared__ double hs[NQ];
+    sum_partials(part, nq, N, hs);
+    if (blockIdx.x == 0 && threadIdx.x < nq)
+        hcol[threadIdx.x] = SECOND ? hcol[threadIdx.x] + hs[threadIdx.x] : hs[threadIdx.x];
+    constexpr int NO = SECOND ? 1 : NQ;
+    double acc[NO];
 #pragma unroll
-    for (int q = 0; q < KRY_MAXM; ++q) {
-        if (q >= nq) break;
-        double v = acc[q];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[wp][q] = v;
+    for (int q = 0; q < NO; ++q) acc[q] = 0.0;
+    for (long i = gs_row(); i < N; i += DOT_BLOCKS * KRY_NT) {
+        double v = w[i];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+            if (q < nq) v -= V[i + ldv * q] * hs[q];
+        w[i] = v;
+        if constexpr (SECOND)
+            acc[0] = fma(v, v, acc[0]);
+        else {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+                if (q < nq) acc[q] = fma(V[i + ldv * q], v, acc[q]);
+        }
     }
-    __syncthreads();
-    for (int q = threadIdx.x; q < nq; q += KRY_NT) {
-        double s = 0.0;
-        for (int k = 0; k < KRY_NT / 32; ++k) s += sh[k][q];
-        partial[(long)blockIdx.x * KRY_MAXM + q] = s;
-    }
+    block_partials<NO>(acc, SECOND ? 1 : nq, N, part2);
 }
 
-// out[q] (= or +=) sum of the partials, q < nq, one warp per q, fixed order.
-__global__ void k_dots_final(const double *__restrict__ partial, int nblk, int nq, double *__restrict__ out,
-                             int accumulate) {
-    pdl_launch_next();
-    pdl_wait_prev();
-    int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (q >= nq) return;
-    double s = 0.0;
-    for (int b = lane; b < nblk; b += 32) s += partial[(long)b * KRY_MAXM + q];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) out[q] = accumulate ? out[q] + s : s;
-}
-
-// w -= V(:, 0:nq) h
-__global__ void k_sub_Vh(const double *__restrict__ V, long ldv, int nq, const double *__restrict__ h,
-                         double *__restrict__ w, long N) {
-    pdl_launch_next();
-    pdl_wait_prev();
-    __shared__ double hs[KRY_MAXM];
-    if (threadIdx.x < nq) hs[threadIdx.x] = h[threadIdx.x];
-    __syncthreads();
-    for (long i = (long)blockIdx.x * KRY_NT + threadIdx.x; i < N; i += (long)gridDim.x * KRY_NT) {
-        double acc = w[i];
-        for (int q = 0; q < nq; ++q) acc -= V[i + ldv * q] * hs[q];
-        w[i] = acc;
-    }
-}
-
-// y = alpha * x / s[0] (s on the device; s[0] == 0 leaves y = 0)
-__global__ void k_scale_by(const double *__restrict__ x, const double *__restrict__ s, double *__restrict__ y,
-                           long N) {
-    pdl_launch_next();
-    pdl_wait_prev();
-    double d = s[0];
-    double inv = d != 0.0 ? 1.0 / d : 0.0;
-    for (long i = (long)blockIdx.x * KRY_NT + threadIdx.x; i < N; i += (long)gridDim.x * KRY_NT) y[i] = x[i] * inv;
-}
-
-__global__ void k_sqrt_into(const double *__restrict__ s2, double *__restrict__ out) {
-    pdl_launch_next();
-    pdl_wait_prev();
-    if (threadIdx.x == 0) out[0] = sqrt(s2[0]);
-}
-
-// r = b - r (r holds A x)
-__global__ void k_resid(const double *__restrict__ b, double *__restrict__ r, long N) {
-    pdl_launch_next();
-    pdl_wait_prev();
-    for (long i = (long)blockIdx.x * KRY_NT + threadIdx.x; i < N; i += (long)gridDim.x * KRY_NT) r[i] = b[i] - r[i];
-}
-
-// Hessenberg column j: apply the earlier rotations, form rotation j, update g.
-// State layout: H (m+1) x m column-major, cs[m], sn[m], g[m+1]; est = |g[j+1]|.
-__global__ void k_givens(double *__restrict__ H, int m, int j, double *__restrict__ cs, double *__restrict__ sn,
-                         double *__restrict__ g, double *__restrict__ est) {
-    pdl_launch_next();
-    pdl_wait_prev();
-    if (threadIdx.x != 0) return;
-    double *h = H + (long)(m + 1) * j;
+// Hessenberg column j (its norm entry c = h[j + 1]): apply the earlier
+// rotations, form rotation j, update g.  State layout: H (m+1) x m column-major,
+// cs[m], sn[m], g[m+1]; est = |g[j+1]|.  One thread.
+__device__ void givens_column(double *__restrict__ h, double c, int j, double *__restrict__ cs,
+                              double *__restrict__ sn, double *__restrict__ g, double *__restrict__ est) {
+    double a = h[0];
     for (int i = 0; i < j; ++i) {
-        double a = h[i], c = h[i + 1];
-        h[i] = cs[i] * a + sn[i] * c;
-        h[i + 1] = -sn[i] * a + cs[i] * c;
+        const double b = h[i + 1], ci = cs[i], si = sn[i];
+        h[i] = ci * a + si * b;
+        a = -si * a + ci * b;
     }
-    double a = h[j], c = h[j + 1];
-    double rr = hypot(a, c);
-    double cj = rr > 0.0 ? a / rr : 1.0, sj = rr > 0.0 ? c / rr : 0.0;
+    const double rr = hypot(a, c);
+    const double cj = rr > 0.0 ? a / rr : 1.0, sj = rr > 0.0 ? c / rr : 0.0;
     cs[j] = cj;
     sn[j] = sj;
     h[j] = rr;
     h[j + 1] = 0.0;
-    g[j + 1] = -sj * g[j];
-    g[j] = cj * g[j];
-    est[0] = fabs(g[j + 1]);
+    const double gj = g[j];
+    g[j + 1] = -sj * gj;
+    g[j] = cj * gj;
+    est[0] = fabs(-sj * gj);
 }
 
-// y = R^-1 g for the leading jend x jend triangle of H
-__global__ void k_backsolve(const double *__restrict__ H, int m, int jend, const double *__restrict__ g,
-                            double *__restrict__ y) {
+// y = x / s (0 where s = 0)
+__device__ __forceinline__ void scale_rows(const double *__restrict__ x, double s, double *__restrict__ y, long N) {
+    const double inv = s != 0.0 ? 1.0 / s : 0.0;
+    for (long i = gs_row(); i < N; i += DOT_BLOCKS * KRY_NT) y[i] = x[i] * inv;
+}
+
+// The end of Arnoldi step j: ||w|| from the partials, the next basis vector,
+// and (one thread) the Hessenberg column and its residual estimate.
+__global__ void __launch_bounds__(GS_NT) k_gs_next(const double *__restrict__ w, long N,
+                                                 const double *__restrict__ part, double *__restrict__ vnext,
+                                                 double *__restrict__ H, int m, int j, double *__restrict__ cs,
+                                                 double *__restrict__ sn, double *__restrict__ g,
+                                                 double *__restrict__ est) {
     pdl_launch_next();
     pdl_wait_prev();
-    if (threadIdx.x != 0) return;
-    for (int i = jend - 1; i >= 0; --i) {
-        double s = g[i];
-        for (int l = i + 1; l < jend; ++l) s -= H[i + (long)(m + 1) * l] * y[l];
-        y[i] = s / H[i + (long)(m + 1) * i];
+    __shared__ double hs[1];
+    sum_partials(part, 1, N, hs);
+    const double nrm = sqrt(hs[0]);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == GS_NT - 1)   // the CTA with the fewest rows
+        givens_column(H + (long)(m + 1) * j, nrm, j, cs, sn, g, est);
+    scale_rows(w, nrm, vnext, N);
+}
+
+// r = b - r (r holds A x); partials of r . r and b . b
+__global__ void __launch_bounds__(GS_NT) k_resid(const double *__restrict__ b, double *__restrict__ r, long N,
+                                               double *__restrict__ part) {
+    pdl_launch_next();
+    pdl_wait_prev();
+    double acc[2] = {0.0, 0.0};
+    for (long i = gs_row(); i < N; i += DOT_BLOCKS * KRY_NT) {
+        const double bi = b[i], v = bi - r[i];
+        r[i] = v;
+        acc[0] = fma(v, v, acc[0]);
+        acc[1] = fma(bi, bi, acc[1]);
     }
+    block_partials<2>(acc, 2, N, part);
 }
 
-// x += Z(:, 0:jend) y
-__global__ void k_update_x(const double *__restrict__ Z, long ldz, int jend, const double *__restrict__ y,
-                           double *__restrict__ x, long N) {
+// nrm = {||r||, ||b||}, V(:, 0) = r / ||r||, g = ||r|| e_1
+__global__ void __launch_bounds__(GS_NT) k_start(const double *__restrict__ r, long N,
+                                               const double *__restrict__ part, double *__restrict__ v0,
+                                               double *__restrict__ g, int m, double *__restrict__ nrm) {
     pdl_launch_next();
     pdl_wait_prev();
-    __shared__ double ys[KRY_MAXM];
-    if (threadIdx.x < jend) ys[threadIdx.x] = y[threadIdx.x];
+    __shared__ double hs[2];
+    sum_partials(part, 2, N, hs);
+    const double beta = sqrt(hs[0]);
+    if (blockIdx.x == 0) {
+        if (threadIdx.x <= m) g[threadIdx.x] = threadIdx.x == 0 ? beta : 0.0;
+        if (threadIdx.x == 0) {
+            nrm[0] = beta;
+            nrm[1] = sqrt(hs[1]);
+        }
+    }
+    scale_rows(r, beta, v0, N);
+}
+
+// x += Z(:, 0:jend) y with y = R^-1 g, R the leading jend x jend triangle of H
+// (solved in every CTA, by one thread from shared memory)
+__global__ void __launch_bounds__(GS_NT) k_update_x(const double *__restrict__ Z, long ldz, int jend,
+                                                  const double *__restrict__ H, int m, const double *__restrict__ g,
+                                                  double *__restrict__ x, long N) {
+    pdl_launch_next();
+    pdl_wait_prev();
+    __shared__ double R[KRY_MAXM][KRY_MAXM + 1], ys[KRY_MAXM];
+    for (int k = threadIdx.x; k < jend * jend; k += GS_NT) R[k % jend][k / jend] = H[k % jend + (long)(m + 1) * (k / jend)];
+    if (threadIdx.x < jend) ys[threadIdx.x] = g[threadIdx.x];
     __syncthreads();
-    for (long i = (long)blockIdx.x * KRY_NT + threadIdx.x; i < N; i += (long)gridDim.x * KRY_NT) {
+    if (threadIdx.x == 0)
+        for (int i = jend - 1; i >= 0; --i) {
+            double s = ys[i];
+            for (int l = i + 1; l < jend; ++l) s -= R[i][l] * ys[l];
+            ys[i] = s / R[i][i];
+        }
+    __syncthreads();
+    for (long i = gs_row(); i < N; i += DOT_BLOCKS * KRY_NT) {
         double acc = x[i];
         for (int q = 0; q < jend; ++q) acc += Z[i + ldz * q] * ys[q];
         x[i] = acc;
     }
 }
 
-__global__ void k_init_g(double *__restrict__ g, int m, const double *__restrict__ beta) {
-    pdl_launch_next();
-    pdl_wait_prev();
-    for (int i = threadIdx.x; i <= m; i += blockDim.x) g[i] = i == 0 ? beta[0] : 0.0;
+// One Arnoldi step's Gram-Schmidt (twice) and its ending: four launches.
+template <int NQ>
+static cudaError_t launch_gs(double *V, long N, int j, double *w, double *part, double *H, int m, double *cs,
+                             double *sn, double *g, double *est, cudaStream_t s) {
+    HSS_PROF("gram_schmidt", s);
+    const dim3 gd(gs_grid(N)), bd(GS_NT);
+    double *part2 = part + DOT_BLOCKS * KRY_MAXM, *hcol = H + (long)(m + 1) * j;
+    cudaError_t e;
+    if ((e = launch_pdl(k_gs_dots<NQ>, gd, bd, 0, s, V, N, j + 1, w, N, part)) ||
+        (e = launch_pdl(k_gs_sub<NQ, false>, gd, bd, 0, s, V, N, j + 1, w, N, part, part2, hcol)) ||
+        (e = launch_pdl(k_gs_sub<NQ, true>, gd, bd, 0, s, V, N, j + 1, w, N, part2, part, hcol)))
+        return e;
+    return launch_pdl(k_gs_next, gd, bd, 0, s, w, N, part, V + N * (j + 1), H, m, j, cs, sn, g, est);
 }
 
 static double spmv_bytes(const hss_bsr *A, int nrhs) {
@@ -320,7 +423,7 @@ int spmv(const hss_bsr *A, int nrhs, const double *x, long ldx, double *y, long 
 
 // Krylov workspace of one solve, carved from the call scratch (cached between calls).
 struct Krylov {
-    ScratchPtr V, Z, w, r, part, H, cs, sn, g, y, scal;
+    ScratchPtr V, Z, w, r, part, H, cs, sn, g, scal;
     int m = 0;
     long N = 0;
     int alloc(Work &W, long n, int mm) {
@@ -328,10 +431,10 @@ struct Krylov {
         if ((rc = W.dalloc_bytes(sizeof(double) * n * (mm + 1), &V.p)) ||
             (rc = W.dalloc_bytes(sizeof(double) * n * mm, &Z.p)) || (rc = W.dalloc_bytes(sizeof(double) * n, &w.p)) ||
             (rc = W.dalloc_bytes(sizeof(double) * n, &r.p)) ||
-            (rc = W.dalloc_bytes(sizeof(double) * DOT_BLOCKS * KRY_MAXM, &part.p)) ||
+            (rc = W.dalloc_bytes(sizeof(double) * 2 * DOT_BLOCKS * KRY_MAXM, &part.p)) ||
             (rc = W.dalloc_bytes(sizeof(double) * (mm + 1) * mm, &H.p)) ||
             (rc = W.dalloc_bytes(sizeof(double) * mm, &cs.p)) || (rc = W.dalloc_bytes(sizeof(double) * mm, &sn.p)) ||
-            (rc = W.dalloc_bytes(sizeof(double) * (mm + 1), &g.p)) || (rc = W.dalloc_bytes(sizeof(double) * mm, &y.p)) ||
+            (rc = W.dalloc_bytes(sizeof(double) * (mm + 1), &g.p)) ||
             (rc = W.dalloc_bytes(sizeof(double) * 8, &scal.p)))
             return rc;
         m = mm;
@@ -342,55 +445,42 @@ struct Krylov {
 
 static thread_local std::vector<std::vector<double>> g_hist;
 
-// sum_i v_i w_i into out[0] (deterministic two-pass)
-static int dot1(const double *v, const double *w, long N, double *part, double *out, int acc, cudaStream_t s) {
-    { HSS_PROF("dots", s); HSS_CUDA(launch_pdl(k_dots, dim3(DOT_BLOCKS), dim3(KRY_NT), 0, s, v, N, 1, w, N, part)); }
-    { HSS_PROF("dots_final", s); HSS_CUDA(launch_pdl(k_dots_final, dim3(1), dim3(32), 0, s, part, DOT_BLOCKS, 1, out, acc)); }
-    HSS_CHECK_LAUNCH("dot");
-    return HSS_OK;
-}
-
 static int fgmres_one(const hss_bsr *A, const Precond &pc, const double *b, double *x, const fgmres_opts &o,
                       Krylov &K, int &iters, double &relres, bool &conv, std::vector<double> &hist, cudaStream_t s) {
     const long N = K.N;
     const int m = K.m;
     double *V = K.V.as<double>(), *Z = K.Z.as<double>(), *w = K.w.as<double>(), *r = K.r.as<double>();
     double *part = K.part.as<double>(), *H = K.H.as<double>(), *sc = K.scal.as<double>();
-    const int gb = DOT_BLOCKS;
+    const dim3 gd(gs_grid(N)), bd(GS_NT);
     int rc;
     double host[2];
-    // ||b||
-    if ((rc = dot1(b, b, N, part, sc + 0, 0, s))) return rc;
-    { HSS_PROF("sqrt_into", s); HSS_CUDA(launch_pdl(k_sqrt_into, dim3(1), dim3(32), 0, s, sc + 0, sc + 1)); }
-    HSS_CUDA(cudaMemcpyAsync(host, sc + 1, sizeof(double), cudaMemcpyDeviceToHost, s));
-    HSS_CUDA(cudaStreamSynchronize(s));
-    const double bnorm = host[0];
+    double bnorm = 0.0;
     iters = 0;
     conv = false;
-    if (bnorm == 0.0) {
-        HSS_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * N, s));
-        relres = 0.0;
-        conv = true;
-        return HSS_OK;
-    }
-    while (true) {
-        // r = b - A x, beta = ||r||
+    for (bool first = true;; first = false) {
+        // r = b - A x, beta = ||r||; the first pass also finds ||b||
         if ((rc = spmv(A, 1, x, N, r, N, s))) return rc;
-        { HSS_PROF("resid", s); HSS_CUDA(launch_pdl(k_resid, dim3(gb), dim3(KRY_NT), 0, s, b, r, N)); }
-        if ((rc = dot1(r, r, N, part, sc + 2, 0, s))) return rc;
-        { HSS_PROF("sqrt_into", s); HSS_CUDA(launch_pdl(k_sqrt_into, dim3(1), dim3(32), 0, s, sc + 2, sc + 3)); }
-        HSS_CUDA(cudaMemcpyAsync(host, sc + 3, sizeof(double), cudaMemcpyDeviceToHost, s));
+        { HSS_PROF("resid", s); HSS_CUDA(launch_pdl(k_resid, gd, bd, 0, s, b, r, N, part)); }
+        { HSS_PROF("start", s); HSS_CUDA(launch_pdl(k_start, gd, bd, 0, s, r, N, part, V, K.g.as<double>(), m, sc)); }
+        HSS_CHECK_LAUNCH("residual");
+        HSS_CUDA(cudaMemcpyAsync(host, sc, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
         HSS_CUDA(cudaStreamSynchronize(s));
-        double beta = host[0];
+        if (first) {
+            bnorm = host[1];
+            if (bnorm == 0.0) {
+                HSS_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * N, s));
+                relres = 0.0;
+                conv = true;
+                return HSS_OK;
+            }
+        }
+        const double beta = host[0];
         relres = beta / bnorm;
         if (relres <= o.rtol) {
             conv = true;
             return HSS_OK;
         }
         if (iters >= o.maxit) return HSS_OK;
-        { HSS_PROF("scale_by", s); HSS_CUDA(launch_pdl(k_scale_by, dim3(gb), dim3(KRY_NT), 0, s, r, sc + 3, V, N)); }
-        { HSS_PROF("init_g", s); HSS_CUDA(launch_pdl(k_init_g, dim3(1), dim3(64), 0, s, K.g.as<double>(), m, sc + 3)); }
-        HSS_CUDA(cudaMemsetAsync(H, 0, sizeof(double) * (m + 1) * m, s));
         int jend = 0;
         for (int j = 0; j < m; ++j) {
             double *vj = V + N * j, *zj = Z + N * j;
@@ -400,21 +490,11 @@ static int fgmres_one(const hss_bsr *A, const Precond &pc, const double *b, doub
                 HSS_CUDA(cudaMemcpyAsync(zj, vj, sizeof(double) * N, cudaMemcpyDeviceToDevice, s));
             }
             if ((rc = spmv(A, 1, zj, N, w, N, s))) return rc;
-            double *hcol = H + (long)(m + 1) * j;
-            // classical Gram-Schmidt, twice
-            for (int pass = 0; pass < 2; ++pass) {
-                { HSS_PROF("dots", s); HSS_CUDA(launch_pdl(k_dots, dim3(gb), dim3(KRY_NT), 0, s, V, N, j + 1, w, N, part)); }
-                { HSS_PROF("dots_final", s); HSS_CUDA(launch_pdl(k_dots_final, dim3(1), dim3(32 * (j + 1)), 0, s, part, gb, j + 1, pass ? K.y.as<double>() : hcol, 0)); }
-                { HSS_PROF("sub_Vh", s); HSS_CUDA(launch_pdl(k_sub_Vh, dim3(gb), dim3(KRY_NT), 0, s, V, N, j + 1, pass ? K.y.as<double>() : hcol, w, N)); }
-            }
-            // h += h2 (the second-pass coefficients, read as a one-block partial sum)
-            { HSS_PROF("dots_final", s); HSS_CUDA(launch_pdl(k_dots_final, dim3(1), dim3(32 * (j + 1)), 0, s, K.y.as<double>(), 1, j + 1, hcol, 1)); }
-            if ((rc = dot1(w, w, N, part, sc + 4, 0, s))) return rc;
-            { HSS_PROF("sqrt_into", s); HSS_CUDA(launch_pdl(k_sqrt_into, dim3(1), dim3(32), 0, s, sc + 4, hcol + j + 1)); }
-            { HSS_PROF("scale_by", s); HSS_CUDA(launch_pdl(k_scale_by, dim3(gb), dim3(KRY_NT), 0, s, w, hcol + j + 1, V + N * (j + 1), N)); }
-            { HSS_PROF("givens", s); HSS_CUDA(launch_pdl(k_givens, dim3(1), dim3(32), 0, s, H, m, j, K.cs.as<double>(), K.sn.as<double>(), K.g.as<double>(), sc + 5)); }
+            // classical Gram-Schmidt, twice; the next basis vector; the rotation
+            auto gs = j < 4 ? launch_gs<4> : j < 8 ? launch_gs<8> : j < 16 ? launch_gs<16> : launch_gs<KRY_MAXM>;
+            HSS_CUDA(gs(V, N, j, w, part, H, m, K.cs.as<double>(), K.sn.as<double>(), K.g.as<double>(), sc + 2, s));
             HSS_CHECK_LAUNCH("arnoldi step");
-            HSS_CUDA(cudaMemcpyAsync(host, sc + 5, sizeof(double), cudaMemcpyDeviceToHost, s));
+            HSS_CUDA(cudaMemcpyAsync(host, sc + 2, sizeof(double), cudaMemcpyDeviceToHost, s));
             HSS_CUDA(cudaStreamSynchronize(s));
             ++iters;
             jend = j + 1;
@@ -422,8 +502,7 @@ static int fgmres_one(const hss_bsr *A, const Precond &pc, const double *b, doub
             hist.push_back(est);
             if (est <= o.rtol || iters >= o.maxit || !(est == est)) break;
         }
-        { HSS_PROF("backsolve", s); HSS_CUDA(launch_pdl(k_backsolve, dim3(1), dim3(32), 0, s, H, m, jend, K.g.as<double>(), K.y.as<double>())); }
-        { HSS_PROF("update_x", s); HSS_CUDA(launch_pdl(k_update_x, dim3(gb), dim3(KRY_NT), 0, s, Z, N, jend, K.y.as<double>(), x, N)); }
+        { HSS_PROF("update_x", s); HSS_CUDA(launch_pdl(k_update_x, gd, bd, 0, s, Z, N, jend, H, m, K.g.as<double>(), x, N)); }
         HSS_CHECK_LAUNCH("fgmres update");
     }
 }
