@@ -8,7 +8,7 @@
 //       x_I = t - W x_B
 // t is parked in a second vector so that all row tiles of a front read the
 // same x_I.  Fronts of one level touch disjoint dofs, so one launch per level
-// covers all of them; each CTA handles APPLY_ROWS rows of one front.
+// covers all of them.
 #include "internal.h"
 #include "front.h"
 #include "factor.h"
@@ -22,14 +22,16 @@
 namespace hssnd {
 
 constexpr int AP_NT = 256;
-constexpr int AP_WPB = AP_NT / 32;   // warps (work items) per CTA
+constexpr int AP_WPB = AP_NT / 32;   // warps per CTA
+constexpr int APPLY_NCH_MAX = 128;   // chunks of a tile at most: 32 KB of FP64 sums
 
-
-// The products of one work item: lane l's sum for row row0 + l.
-template <class T, bool FWD>
-__device__ __forceinline__ T apply_item_sum(const ApplyItem &it, const FrontDev &F, const T *__restrict__ arena,
-                                            const int *__restrict__ iperm, const int *__restrict__ blist,
-                                            const double *__restrict__ w) {
+// The products of columns [c0, c1) of a 32-row tile: lane l's sum for row
+// row0 + l.  after_wait() runs once, when the previous kernel's vectors are there.
+template <class T, bool FWD, class AfterWait>
+__device__ __forceinline__ T apply_item_sum(const ApplyItem &it, int c0, int c1, const FrontDev &F,
+                                            const T *__restrict__ arena, const int *__restrict__ iperm,
+                                            const int *__restrict__ blist, const double *w, bool &waited,
+                                            AfterWait &&after_wait) {
     const int lane = threadIdx.x & 31;
     const T *M = arena + F.foff;
     const int colbase = FWD ? 0 : F.ni, nrows = FWD ? F.n : F.ni;
@@ -38,17 +40,17 @@ __device__ __forceinline__ T apply_item_sum(const ApplyItem &it, const FrontDev 
     // arithmetic in the factor's precision (FP32 factors: FP32 products and sums;
     // GB300's FP64 pipe is a small fraction of its FP32 rate)
     T acc = T(0);
-    bool waited = false;
-    for (int cg = it.c0; cg < it.c1; cg += 32) {
+    for (int cg = c0; cg < c1; cg += 32) {
         const int c = cg + lane;
         T m[32];
         const T *col = M + i + (long)F.n * (colbase + cg);
 #pragma unroll
-        for (int q = 0; q < 32; ++q) m[q] = (rowok && cg + q < it.c1) ? col[(long)F.n * q] : T(0);
-        const int dof = c < it.c1 ? (FWD ? iperm[F.iperm_off + c] : blist[F.bset_off + c]) : -1;
+        for (int q = 0; q < 32; ++q) m[q] = (rowok && cg + q < c1) ? col[(long)F.n * q] : T(0);
+        const int dof = c < c1 ? (FWD ? iperm[F.iperm_off + c] : blist[F.bset_off + c]) : -1;
         if (!waited) {   // the vectors are the previous kernel's output
             pdl_wait_prev();
             waited = true;
+            after_wait();
         }
         const T z = dof >= 0 ? (T)w[dof] : T(0);
 #pragma unroll
@@ -57,183 +59,213 @@ __device__ __forceinline__ T apply_item_sum(const ApplyItem &it, const FrontDev 
     return acc;
 }
 
-// The result of one work item (row row0 + lane):
-//   FWD: rows [0, ni) to t, rows [ni, n) added into x_B;  BWD: x_I = t - sum
-template <class T, bool FWD>
-__device__ __forceinline__ void apply_item_store(const ApplyItem &it, const FrontDev &F, const int *__restrict__ ilist,
-                                                 const int *__restrict__ blist, double *__restrict__ w,
-                                                 double *__restrict__ tv, T acc) {
+// The dof that lane l of a tile writes (row row0 + l; -1 past the last row), and
+// its result: FWD: rows [0, ni) to t, rows [ni, n) added into x_B;  BWD: x_I = t - sum
+// (old: the value of x_B or t before).
+template <bool FWD>
+__device__ __forceinline__ int apply_dof(const ApplyItem &it, const FrontDev &F, const int *__restrict__ ilist,
+                                         const int *__restrict__ blist) {
     const int i = it.row0 + (threadIdx.x & 31);
-    if (i >= (FWD ? F.n : F.ni)) return;
-    const double y = (double)acc;
-    if (FWD) {
-        if (i < F.ni)
-            tv[ilist[F.iset_off + i]] = y;
-        else
-            w[blist[F.bset_off + i - F.ni]] += y;
-    } else {
-        const int dof = ilist[F.iset_off + i];
-        w[dof] = tv[dof] - y;
-    }
+    if (i >= (FWD ? F.n : F.ni)) return -1;
+    return i < F.ni ? ilist[F.iset_off + i] : blist[F.bset_off + i - F.ni];
+}
+template <bool FWD>
+__device__ __forceinline__ double apply_old(const ApplyItem &it, const FrontDev &F, int dof, const double *w,
+                                            const double *tv) {
+    if (FWD) return dof >= 0 && it.row0 + (int)(threadIdx.x & 31) >= F.ni ? w[dof] : 0.0;
+    return dof >= 0 ? tv[dof] : 0.0;
+}
+template <bool FWD>
+__device__ __forceinline__ void apply_store(const ApplyItem &it, const FrontDev &F, int dof, double old, double y,
+                                            double *w, double *tv) {
+    if (dof < 0) return;
+    if (!FWD)
+        w[dof] = old - y;
+    else if (it.row0 + (int)(threadIdx.x & 31) < F.ni)
+        tv[dof] = y;
+    else
+        w[dof] = old + y;
 }
 
-// One vector (several: apply_multi.cu).  One warp per work item = (front,
-// 32-row tile, column chunk of at most APPLY_CHUNK columns).  Lane l owns row
-// row0 + l; x is gathered one value per lane and broadcast by shuffles; 32
-// matrix loads per lane are in flight per group of 32 columns.  A tile split
-// over several chunks writes partial sums; the last warp to finish (atomic
-// ticket) adds them in chunk order and writes the result, so the sum order is
-// fixed.  No barrier, no waiting.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// p's counterpart in the cluster's first CTA
+template <class T> __device__ __forceinline__ void store_first_cta(T *p, T v) {
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(a));
+    if constexpr (sizeof(T) == 8)
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+    else
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r), "f"(v) : "memory");
+}
+
+// One vector (several: apply_multi.cu).  A 32-row tile of a front is the work of
+// `slots` warps: warp k takes the column chunks k, k + slots, ... of `chunk`
+// columns, lane l owning row row0 + l; x is gathered one value per lane and
+// broadcast by shuffles; 32 matrix loads per lane are in flight before the wait
+// for the previous level.  The warps leave their sums in the shared memory of
+// the tile's (first) CTA, and one warp adds them in chunk order, so the sum order
+// is fixed.  CL = 1: slots <= 8, and a CTA holds 8 / slots tiles; else a cluster
+// of CL CTAs shares one tile.  A level is one chain of latencies (wait, gather,
+// products, sum, store), so partial sums meet in shared memory, not behind a
+// device-wide ticket and a second read (two L2 round trips), and what the store
+// adds to is loaded with the gather.  64 x 64 quads, p = 2, 21 level launches:
+// FP32 (106 MB) 106 -> 71 us, FP64 (208 MB) 197 -> 157 us, of which the FP64 pipe
+// takes 41.  The deepest levels walked by one launch of a CTA per subtree were
+// slower than this kernel's levels (FP32 82, FP64 162 us).
 //   FWD: y = [F_ii^-1 P^t ; -F_bi F_ii^-1 P^t] x(Iperm)  ->  t = y[0,ni), x_B += y[ni,n)
 //   BWD: x_I = t - W x_B
-template <class T, bool FWD>
-__global__ void __launch_bounds__(AP_NT) k_apply(const ApplyItem *__restrict__ items, int nitems,
+template <class T, bool FWD, int CL>
+__global__ void __launch_bounds__(AP_NT) k_apply(const ApplyItem *__restrict__ tiles, int ntiles, ApplyShape sh,
                                                const FrontDev *__restrict__ fr, const T *__restrict__ arena,
                                                const int *__restrict__ iperm, const int *__restrict__ ilist,
-                                               const int *__restrict__ blist, const ApplyParams *__restrict__ prm,
-                                               double *__restrict__ part, int *__restrict__ tickets) {
+                                               const int *__restrict__ blist, const ApplyParams *__restrict__ prm) {
     pdl_launch_next();
-    const int lane = threadIdx.x & 31;
-    const int item = blockIdx.x * AP_WPB + (threadIdx.x >> 5);
-    if (item >= nitems) return;   // whole warps leave together
-    const ApplyItem it = items[item];
-    const FrontDev F = fr[it.front];
-    T acc = apply_item_sum<T, FWD>(it, F, arena, iperm, blist, prm->w);
-    pdl_wait_prev();   // (an item without columns has not waited yet)
-    if (it.nchunk > 1) {
-        reinterpret_cast<T *>(part)[(long)item * 32 + lane] = acc;
-        __threadfence();
-        int ticket = 0;
-        if (lane == 0) ticket = atomicAdd(&tickets[it.tile], 1);
-        ticket = __shfl_sync(0xffffffffu, ticket, 0);
-        if (ticket != it.nchunk - 1) return;
-        __threadfence();
-        const T *first = reinterpret_cast<const T *>(part) + (long)it.first * 32;
+    if constexpr (CL > 1) cluster_arrive();
+    extern __shared__ __align__(16) unsigned char apply_smem[];   // [tiles of the CTA][sh.nch][32]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lt = CL > 1 ? 0 : warp / sh.slots;
+    const int slot = CL > 1 ? (int)(blockIdx.x % CL) * (int)(blockDim.x / 32) + warp : warp % sh.slots;
+    const int tile = CL > 1 ? (int)(blockIdx.x / CL) : (int)blockIdx.x * sh.per + lt;
+    T *sums = reinterpret_cast<T *>(apply_smem) + (long)lt * sh.nch * 32 + lane;
+    const bool on = tile < ntiles, writer = on && slot == 0;
+    ApplyItem it{};
+    FrontDev F{};
+    double *w = prm->w, *tv = prm->tv;
+    int nch = 0, dof = -1;
+    if (on) {
+        it = tiles[tile];
+        F = fr[it.front];
+        nch = max(1, (it.c1 + sh.chunk - 1) / sh.chunk);
+        if (writer) dof = apply_dof<FWD>(it, F, ilist, blist);
+    }
+    double old = 0.0;
+    T acc = T(0);
+    bool waited = false, started = false;
+    for (int ch = slot; ch < nch; ch += sh.slots) {
+        acc = apply_item_sum<T, FWD>(it, ch * sh.chunk, min(it.c1, (ch + 1) * sh.chunk), F, arena, iperm, blist, w,
+                                     waited, [&] { old = apply_old<FWD>(it, F, dof, w, tv); });
+        if (sh.nch > 1) {
+            if constexpr (CL > 1) {
+                if (!started) cluster_wait();   // the first CTA runs
+                started = true;
+                store_first_cta(sums + ch * 32, acc);
+            } else
+                sums[ch * 32] = acc;
+        }
+    }
+    if (!waited) {   // (no columns)
+        pdl_wait_prev();
+        old = apply_old<FWD>(it, F, dof, w, tv);
+    }
+    if (sh.nch > 1) {
+        if constexpr (CL > 1) {
+            if (!started) cluster_wait();
+            cluster_arrive();
+            cluster_wait();
+        } else
+            __syncthreads();
+        if (!writer) return;
         acc = T(0);
-        for (int ch = 0; ch < it.nchunk; ++ch) acc += __ldcg(first + (long)ch * 32 + lane);
-        if (lane == 0) tickets[it.tile] = 0;   // ready for the next apply
+        for (int ch = 0; ch < nch; ++ch) acc += sums[ch * 32];
     }
-    apply_item_store<T, FWD>(it, F, ilist, blist, prm->w, prm->tv, acc);
+    if (writer) apply_store<FWD>(it, F, dof, old, (double)acc, w, tv);
 }
 
-// The deepest levels as one launch: CTA s walks the stages of subtree s (the
-// fronts below its root in stage nst - 1), deepest stage first forward and
-// root first backward, its eight warps taking the stage's items (one 32-row
-// tile, every column) and a block barrier between stages.  Subtrees hold
-// disjoint dofs (DG dofs belong to elements), so the CTAs never meet; inside
-// one, the barrier orders a stage's writes of x before the next stage's reads.
-template <class T, bool FWD>
-__global__ void __launch_bounds__(AP_NT) k_apply_sub(const ApplyItem *__restrict__ items, const int *__restrict__ off,
-                                                   int nst, const FrontDev *__restrict__ fr, const T *__restrict__ arena,
-                                                   const int *__restrict__ iperm, const int *__restrict__ ilist,
-                                                   const int *__restrict__ blist, const ApplyParams *__restrict__ prm) {
-    pdl_launch_next();
-    const int sub = blockIdx.x, warp = threadIdx.x >> 5;
-    double *w = prm->w;
-    double *tv = prm->tv;
-    for (int l = 0; l < nst; ++l) {
-        const int q = FWD ? l : nst - 1 - l;
-        const int b = off[sub * (nst + 1) + q], e = off[sub * (nst + 1) + q + 1];
-        for (int k = b + warp; k < e; k += AP_WPB) {
-            const ApplyItem it = items[k];
-            const FrontDev F = fr[it.front];
-            const T acc = apply_item_sum<T, FWD>(it, F, arena, iperm, blist, w);
-            pdl_wait_prev();
-            apply_item_store<T, FWD>(it, F, ilist, blist, w, tv, acc);
-        }
-        pdl_wait_prev();   // warps without items
-        __syncthreads();
-    }
-}
-
-__global__ void k_apply_set(ApplyParams *d, ApplyParams v) {
+// The arguments for the sweep's kernels, and w = x (every right-hand side)
+// unless they alias.
+__global__ void k_apply_begin(ApplyParams *d, ApplyParams v, long N) {
     if (threadIdx.x == 0 && blockIdx.x == 0) *d = v;
-}
-
-// w = x (every right-hand side), skipped when they alias
-__global__ void k_apply_copyin(const ApplyParams *__restrict__ prm, long N) {
-    pdl_launch_next();
-    const double *x = prm->x;
-    double *w = prm->w;
-    if (x == w) return;
-    long tot = N * prm->nrhs;
+    if (v.x == v.w) return;
+    const long tot = N * v.nrhs;
     for (long g = (long)blockIdx.x * blockDim.x + threadIdx.x; g < tot; g += (long)gridDim.x * blockDim.x) {
-        long r = g / N, i = g % N;
-        w[i + prm->ldw * r] = x[i + prm->ldx * r];
+        const long r = g / N, i = g % N;
+        v.w[i + v.ldw * r] = v.x[i + v.ldx * r];
     }
 }
 
-// The whole sweep (copy-in, forward levels, top block, backward levels) as
-// one kernel sequence on stream s, each launch overlapping the previous one's
-// tail (launch_pdl); parameters come from f->d_aparams.  RB = 1: one vector;
-// else up to RB, every level in a launch of its own.
+// How many chunks the widest tile of a level has, and the warps and CTAs a tile
+// gets: a warp per chunk (no idle ones: a level's warps compete for the SMs'
+// registers), up to 8 CTAs of 8 (the portable cluster size).
+static ApplyShape apply_shape(int ncols, int chunk) {
+    ApplyShape sh;
+    sh.chunk = chunk;
+    while (cdiv(ncols, sh.chunk) > APPLY_NCH_MAX) sh.chunk *= 2;
+    sh.nch = std::max(1, cdiv(ncols, sh.chunk));
+    while (sh.cl < 8 && sh.nch > sh.cl * AP_WPB) sh.cl *= 2;
+    sh.slots = sh.cl * std::min(AP_WPB, cdiv(sh.nch, sh.cl));
+    sh.per = std::max(1, AP_WPB / sh.slots);
+    return sh;
+}
+
+template <class T, bool FWD>
+static cudaError_t launch_apply(const hss_factor_t *f, const ApplyStage &st, cudaStream_t s) {
+    const ApplyShape &sh = st.shape[FWD ? 0 : 1];
+    const int nt = FWD ? st.nfwd : st.nbwd;
+    auto kern = sh.cl == 1   ? k_apply<T, FWD, 1>
+                : sh.cl == 2 ? k_apply<T, FWD, 2>
+                : sh.cl == 4 ? k_apply<T, FWD, 4>
+                             : k_apply<T, FWD, 8>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cdiv(nt, sh.per) * sh.cl);
+    cfg.blockDim = dim3(32 * sh.per * sh.slots / sh.cl);
+    cfg.dynamicSmemBytes = sh.nch > 1 ? sizeof(T) * 32 * sh.nch * sh.per : 0;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_pdl
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = sh.cl;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = sh.cl > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, (const ApplyItem *)(FWD ? st.d_fwd : st.d_bwd), nt, sh,
+                              (const FrontDev *)st.d_fronts, f->arena_ptr<T>(), (const int *)f->d_iperm.as<int>(),
+                              (const int *)(st.top ? f->d_topset.as<int>() : f->tree->d_iset.as<int>()),
+                              (const int *)f->tree->d_bset.as<int>(), (const ApplyParams *)f->d_aparams.as<ApplyParams>());
+}
+
+// The whole sweep (forward levels, top block, backward levels) as one kernel
+// sequence on stream s, each launch overlapping the previous one's tail
+// (launch_pdl); parameters come from f->d_aparams.  RB = 1: one vector; else up
+// to RB.
 template <class T, int RB> static int record_sweep(const hss_factor_t *f, cudaStream_t s, int &nk) {
-    const T *arena = f->arena_ptr<T>();
-    const ApplyParams *prm = f->d_aparams.as<ApplyParams>();
-    const int *iperm = f->d_iperm.as<int>(), *blist = f->tree->d_bset.as<int>();
     nk = 0;
-    k_apply_copyin<<<2 * device_sms(), 256, 0, s>>>(prm, f->ndof);
-    ++nk;
     cudaError_t e = cudaSuccess;
-    const int sub_nst = RB == 1 ? f->sub_nst : 0;
-    auto sub = [&](bool fwd) {
-        if constexpr (RB == 1) {
-            if (sub_nst == 0 || e != cudaSuccess) return;
-            e = launch_pdl(fwd ? k_apply_sub<T, true> : k_apply_sub<T, false>, dim3(f->sub_n), dim3(AP_NT), 0, s,
-                           (const ApplyItem *)(fwd ? f->d_sub_fwd : f->d_sub_bwd),
-                           (const int *)(fwd ? f->d_sub_off_fwd : f->d_sub_off_bwd), sub_nst,
-                           (const FrontDev *)f->d_sub_fronts, arena, iperm, (const int *)f->tree->d_iset.as<int>(), blist,
-                           prm);
-            ++nk;
-        }
-    };
     for (int pass = 0; pass < 2; ++pass) {
         const bool fwd = pass == 0;
-        if (fwd) sub(true);
         for (size_t k = 0; k < f->apply.size(); ++k) {
             const size_t q = fwd ? k : f->apply.size() - 1 - k;
-            if ((int)q < sub_nst) continue;   // in the subtree launch
             const ApplyStage &st = f->apply[q];
-            const int *ilist = st.top ? f->d_topset.as<int>() : f->tree->d_iset.as<int>();
-            const int nt = fwd ? st.nfwd : st.nbwd;
-            if (nt == 0) continue;
+            if ((fwd ? st.nfwd : st.nbwd) == 0) continue;
             if (e != cudaSuccess) break;
             if constexpr (RB > 1)
                 e = launch_apply_multi<T, RB>(f, q, fwd, s);
             else
-                e = launch_pdl(fwd ? k_apply<T, true> : k_apply<T, false>, dim3(cdiv(nt, AP_WPB)), dim3(AP_NT), 0, s,
-                               (const ApplyItem *)(fwd ? st.d_fwd : st.d_bwd), nt, (const FrontDev *)st.d_fronts, arena,
-                               iperm, ilist, blist, prm,
-                               f->d_apart.as<double>() + (fwd ? st.part_fwd : st.part_bwd) * 32,
-                               f->d_tickets.as<int>() + (fwd ? st.tk_fwd : st.tk_bwd));
+                e = fwd ? launch_apply<T, true>(f, st, s) : launch_apply<T, false>(f, st, s);
             ++nk;
         }
-        if (!fwd) sub(false);
     }
     if (e != cudaSuccess) return cuda_fail(e, "apply sweep launch");
     HSS_CHECK_LAUNCH("apply sweep");
     return HSS_OK;
 }
 
-// Work items of one sweep direction of a stage: 32-row tiles, each split into
-// column chunks of `chunk` (pass 0: forward, n rows x ni columns; pass 1:
-// backward, ni rows x nb columns).
-static void stage_items(const ApplyStage &st, int pass, int chunk, std::vector<ApplyItem> &items, int &tiles) {
+// The 32-row tiles of one sweep direction of a stage (pass 0: forward, n rows x
+// ni columns; pass 1: backward, ni rows x nb columns), each with every column.
+static int stage_items(const ApplyStage &st, int pass, std::vector<ApplyItem> &items) {
+    int ncmax = 0;
     items.clear();
-    tiles = 0;
     for (int f = 0; f < (int)st.h_fronts.size(); ++f) {
         const FrontDev &d = st.h_fronts[f];
         if (d.ni == 0) continue;
         const int nrows = pass == 0 ? d.n : d.ni;
         const int ncols = pass == 0 ? d.ni : d.nb;
-        const int nch = std::max(1, cdiv(ncols, chunk));
-        for (int r0 = 0; r0 < nrows; r0 += 32) {
-            const int first = (int)items.size();
-            const int tile = nch > 1 ? tiles++ : -1;
-            for (int ch = 0; ch < nch; ++ch)
-                items.push_back({f, r0, std::min(ncols, ch * chunk), std::min(ncols, (ch + 1) * chunk), tile, first, nch});
-        }
+        ncmax = std::max(ncmax, ncols);
+        for (int r0 = 0; r0 < nrows; r0 += 32) items.push_back({f, r0, 0, ncols, -1, (int)items.size(), 1});
     }
+    return ncmax;
 }
 
 int pack_apply(hss_factor_t *F, cudaStream_t s) {
@@ -244,89 +276,18 @@ int pack_apply(hss_factor_t *F, cudaStream_t s) {
         }
     const size_t nst = F->apply.size();
     std::vector<std::vector<ApplyItem>> items(2 * nst);
-    long part_total = 0;
-    int tk_total = 0;
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
     size_t bytes = 0;
     for (size_t q = 0; q < nst; ++q) {
         ApplyStage &st = F->apply[q];
-        int tiles[2];
-        for (int pass = 0; pass < 2; ++pass) stage_items(st, pass, st.chunk[pass], items[2 * q + pass], tiles[pass]);
+        for (int pass = 0; pass < 2; ++pass) {
+            st.shape[pass] = apply_shape(stage_items(st, pass, items[2 * q + pass]), st.chunk[pass]);
+            st.chunk[pass] = st.shape[pass].chunk;
+        }
         st.nfwd = (int)items[2 * q].size();
         st.nbwd = (int)items[2 * q + 1].size();
-        st.part_fwd = part_total;
-        part_total += st.nfwd;
-        st.part_bwd = part_total;
-        part_total += st.nbwd;
-        st.tk_fwd = tk_total;
-        tk_total += tiles[0];
-        st.tk_bwd = tk_total;
-        tk_total += tiles[1];
         bytes += al(sizeof(FrontDev) * st.h_fronts.size()) + al(sizeof(ApplyItem) * st.nfwd) +
                  al(sizeof(ApplyItem) * st.nbwd);
-    }
-    // subtree part: root stage = the shallowest stage (below the top block)
-    // with at least APPLY_SUB_MIN fronts, none larger than APPLY_SUB_MAXN
-    // (this and every deeper stage); every front of the stages up to it
-    // belongs to the subtree of its ancestor in the root stage
-    int qr = -1;
-    for (size_t q = 0; q < nst; ++q) {
-        if (F->apply[q].top) break;
-        int nmax = 0;
-        for (const FrontDev &d : F->apply[q].h_fronts) nmax = std::max(nmax, d.n);
-        if (nmax > APPLY_SUB_MAXN) break;   // larger fronts need the level launch's parallelism
-        if (F->apply[q].nfronts >= APPLY_SUB_MIN) qr = (int)q;
-    }
-    std::vector<FrontDev> sfr;
-    std::vector<ApplyItem> sit[2];
-    std::vector<int> soff[2];
-    F->sub_nst = 0;
-    F->sub_n = 0;
-    if (qr >= 1) {
-        const hss_tree *t = F->tree;
-        const int nsub = (int)F->apply[qr].h_fronts.size();
-        const int root_level = t->level[F->apply[qr].h_fronts[0].box];
-        std::unordered_map<int, int> sub_of_root;
-        for (int f = 0; f < nsub; ++f) sub_of_root[F->apply[qr].h_fronts[f].box] = f;
-        // per subtree and stage, its fronts
-        std::vector<std::vector<int>> lists((size_t)nsub * (qr + 1));
-        for (int q = 0; q <= qr; ++q) {
-            const ApplyStage &st = F->apply[q];
-            for (int f = 0; f < (int)st.h_fronts.size(); ++f) {
-                int b = st.h_fronts[f].box;
-                while (b >= 0 && t->level[b] > root_level) b = t->parent[b];
-                const auto it = sub_of_root.find(b);
-                if (it == sub_of_root.end()) {   // not below a root (cannot happen in a box tree)
-                    qr = -1;
-                    break;
-                }
-                lists[(size_t)it->second * (qr + 1) + q].push_back((int)sfr.size());
-                sfr.push_back(st.h_fronts[f]);
-            }
-            if (qr < 0) break;
-        }
-        if (qr >= 1) {
-            for (int pass = 0; pass < 2; ++pass) {
-                soff[pass].assign((size_t)nsub * (qr + 2), 0);
-                for (int sb = 0; sb < nsub; ++sb)
-                    for (int q = 0; q <= qr; ++q) {
-                        soff[pass][(size_t)sb * (qr + 2) + q] = (int)sit[pass].size();
-                        for (int fi : lists[(size_t)sb * (qr + 1) + q]) {
-                            const FrontDev &d = sfr[fi];
-                            if (d.ni == 0) continue;
-                            const int nrows = pass == 0 ? d.n : d.ni, ncols = pass == 0 ? d.ni : d.nb;
-                            for (int r0 = 0; r0 < nrows; r0 += 32)
-                                sit[pass].push_back({fi, r0, 0, ncols, -1, (int)sit[pass].size(), 1});
-                        }
-                        soff[pass][(size_t)sb * (qr + 2) + q + 1] = (int)sit[pass].size();
-                    }
-            }
-            F->sub_nst = qr + 1;
-            F->sub_n = nsub;
-            bytes += al(sizeof(FrontDev) * sfr.size()) + al(sizeof(ApplyItem) * sit[0].size()) +
-                     al(sizeof(ApplyItem) * sit[1].size()) + al(sizeof(int) * soff[0].size()) +
-                     al(sizeof(int) * soff[1].size());
-        }
     }
     // every stage's fronts and work items in one device allocation
     std::vector<char> pack(std::max(bytes, (size_t)1));
@@ -346,18 +307,7 @@ int pack_apply(hss_factor_t *F, cudaStream_t s) {
         st.d_fwd = reinterpret_cast<ApplyItem *>(put(items[2 * q].data(), sizeof(ApplyItem) * st.nfwd));
         st.d_bwd = reinterpret_cast<ApplyItem *>(put(items[2 * q + 1].data(), sizeof(ApplyItem) * st.nbwd));
     }
-    if (F->sub_nst > 0) {
-        F->d_sub_fronts = reinterpret_cast<FrontDev *>(put(sfr.data(), sizeof(FrontDev) * sfr.size()));
-        F->d_sub_fwd = reinterpret_cast<ApplyItem *>(put(sit[0].data(), sizeof(ApplyItem) * sit[0].size()));
-        F->d_sub_bwd = reinterpret_cast<ApplyItem *>(put(sit[1].data(), sizeof(ApplyItem) * sit[1].size()));
-        F->d_sub_off_fwd = reinterpret_cast<int *>(put(soff[0].data(), sizeof(int) * soff[0].size()));
-        F->d_sub_off_bwd = reinterpret_cast<int *>(put(soff[1].data(), sizeof(int) * soff[1].size()));
-    }
     HSS_CUDA(cudaMemcpyAsync(base, pack.data(), pack.size(), cudaMemcpyHostToDevice, s));
-    if ((rc = F->d_apart.alloc(sizeof(double) * 32 * std::max(part_total, 1L))) ||
-        (rc = F->d_tickets.alloc(sizeof(int) * std::max(tk_total, 1))))
-        return rc;
-    HSS_CUDA(cudaMemsetAsync(F->d_tickets.p, 0, sizeof(int) * std::max(tk_total, 1), s));
     // (a copy from pageable memory has left `pack` by the time cudaMemcpyAsync returns)
     return HSS_OK;
 }
@@ -366,10 +316,7 @@ int pack_apply(hss_factor_t *F, cudaStream_t s) {
 // captured graph for one right-hand side); ms[2 * q + pass] = that launch's time.
 template <class T> static int timed_sweep(const hss_factor_t *f, cudaStream_t s, std::vector<cudaEvent_t> &ev,
                                           std::vector<float> &ms) {
-    const T *arena = f->arena_ptr<T>();
-    const ApplyParams *prm = f->d_aparams.as<ApplyParams>();
     const size_t nst = f->apply.size();
-    k_apply_copyin<<<2 * device_sms(), 256, 0, s>>>(prm, f->ndof);
     for (int pass = 0; pass < 2; ++pass) {
         const bool fwd = pass == 0;
         for (size_t k = 0; k < nst; ++k) {
@@ -377,18 +324,8 @@ template <class T> static int timed_sweep(const hss_factor_t *f, cudaStream_t s,
             const ApplyStage &st = f->apply[q];
             const int nt = fwd ? st.nfwd : st.nbwd;
             if (nt == 0) continue;
-            const int *ilist = st.top ? f->d_topset.as<int>() : f->tree->d_iset.as<int>();
-            double *part = f->d_apart.as<double>() + (fwd ? st.part_fwd : st.part_bwd) * 32;
-            int *tk = f->d_tickets.as<int>() + (fwd ? st.tk_fwd : st.tk_bwd);
             HSS_CUDA(cudaEventRecord(ev[2 * (2 * q + pass)], s));
-            if (fwd)
-                k_apply<T, true><<<cdiv(nt, AP_WPB), AP_NT, 0, s>>>(st.d_fwd, nt, st.d_fronts, arena,
-                                                                       f->d_iperm.as<int>(), ilist,
-                                                                       f->tree->d_bset.as<int>(), prm, part, tk);
-            else
-                k_apply<T, false><<<cdiv(nt, AP_WPB), AP_NT, 0, s>>>(st.d_bwd, nt, st.d_fronts, arena,
-                                                                        f->d_iperm.as<int>(), ilist,
-                                                                        f->tree->d_bset.as<int>(), prm, part, tk);
+            HSS_CUDA((fwd ? launch_apply<T, true>(f, st, s) : launch_apply<T, false>(f, st, s)));
             HSS_CUDA(cudaEventRecord(ev[2 * (2 * q + pass) + 1], s));
         }
     }
@@ -448,8 +385,8 @@ int tune_apply(hss_factor_t *F, cudaStream_t s) {
     HSS_CUDA(cudaMemsetAsync(F->tvec.p, 0, sizeof(double) * F->ndof, s));
     ApplyParams pv{yb.as<double>(), (long)F->ndof, yb.as<double>(), (long)F->ndof, F->tvec.as<double>(),
                    (long)F->ndof, 1};
-    k_apply_set<<<1, 32, 0, s>>>(F->d_aparams.as<ApplyParams>(), pv);
-    HSS_CHECK_LAUNCH("k_apply_set");
+    k_apply_begin<<<1, 32, 0, s>>>(F->d_aparams.as<ApplyParams>(), pv, (long)F->ndof);
+    HSS_CHECK_LAUNCH("k_apply_begin");
     std::vector<cudaEvent_t> ev(4 * nst, nullptr);
     for (auto &e : ev) HSS_CUDA(cudaEventCreate(&e));
     std::vector<float> best(2 * nst, 1e30f), ms(2 * nst, 0.f);
@@ -525,8 +462,8 @@ int apply_factor(const hss_factor_t *f, int nrhs, const double *x, long ldx, dou
         }
         ApplyParams pv{x + ldx * k, ldx, y + ldy * k, ldy, mf->tvec.as<double>(), (long)f->ndof, nr};
         prof_add_launches(f->graph_kernels[slot]);
-        k_apply_set<<<1, 32, 0, s>>>(mf->d_aparams.as<ApplyParams>(), pv);
-        HSS_CHECK_LAUNCH("k_apply_set");
+        k_apply_begin<<<2 * device_sms(), 256, 0, s>>>(mf->d_aparams.as<ApplyParams>(), pv, (long)f->ndof);
+        HSS_CHECK_LAUNCH("k_apply_begin");
         HSS_CUDA(cudaGraphLaunch(f->gexec[slot], s));
     }
     return HSS_OK;

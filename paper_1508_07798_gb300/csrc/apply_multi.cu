@@ -277,7 +277,7 @@ cudaError_t launch_apply_multi(const hss_factor_t *F, size_t q, bool fwd, cudaSt
     const FrontDev *fr = st.d_fronts;
     const T *arena = F->arena_ptr<T>();
     const ApplyParams *prm = F->d_aparams.as<ApplyParams>();
-    const int seg = (int)q < F->sub_nst ? 1 << 30 : st.chunk[pass];   // (a subtree's item holds every column)
+    const int seg = st.chunk[pass];
     if (fwd)
         return launch_pdl(k_apply_multi<T, RB, true>, dim3(m.cnt[pass]), dim3(MA_NT), 0, s, items, fr, arena, ip, il, bl,
                           prm, part, tk, seg);

@@ -7,11 +7,7 @@
 
 namespace hssnd {
 
-constexpr int APPLY_ROWS = 32;
-
-constexpr int APPLY_CHUNK = 64;   // columns per warp work item of the apply
-constexpr int APPLY_SUB_MIN = 256;   // fronts of the level that roots the apply's subtrees (one CTA each)
-constexpr int APPLY_SUB_MAXN = 192;  // largest front (n) of the levels the subtree launch takes
+constexpr int APPLY_CHUNK = 64;   // columns per warp of the apply
 
 struct ApplyItem {
     int front;        // stage-local front index
@@ -29,17 +25,22 @@ struct ApplyMultiStage {
     int off[2], cnt[2], tk[2];
 };
 
+// One level launch of the single-vector apply: columns per chunk, the most
+// chunks of a tile, the warps of a tile, and the CTAs of a tile or the tiles of a CTA.
+struct ApplyShape {
+    int chunk = APPLY_CHUNK, nch = 1, slots = 1, cl = 1, per = 1;
+};
+
 // Per level (and the top block): fronts and the row tiles of the apply.
 struct ApplyStage {
     bool top = false;
     int nfronts = 0;
     std::vector<FrontDev> h_fronts;       // host copies, packed into the factor's apply buffer
-    int chunk[2] = {APPLY_CHUNK, APPLY_CHUNK};   // columns per work item of the forward / backward sweep
+    int chunk[2] = {APPLY_CHUNK, APPLY_CHUNK};   // columns per warp of the forward / backward sweep
     FrontDev *d_fronts = nullptr;
     ApplyItem *d_fwd = nullptr, *d_bwd = nullptr;
-    int nfwd = 0, nbwd = 0;               // work items (warps) of the two sweeps
-    long part_fwd = 0, part_bwd = 0;      // offsets (in items) into the partial-sum buffer
-    int tk_fwd = 0, tk_bwd = 0;           // offsets into the ticket array
+    int nfwd = 0, nbwd = 0;               // row tiles of the two sweeps
+    ApplyShape shape[2];                  // their warps and CTAs
     double fwd_bytes = 0, bwd_bytes = 0;  // factor entries read (x8 bytes in FP64)
     double fwd_vec = 0, bwd_vec = 0;      // vector entries read + written per right-hand side
 };
@@ -129,16 +130,7 @@ struct hss_factor_t {
     std::vector<hssnd::ApplyMultiStage> multi;   // per stage, filled by the first apply to several vectors
     hssnd::DevBuf multi_items, multi_tickets, multi_part;
     hssnd::DevBuf d_aparams;
-    hssnd::DevBuf d_apart;       // partial sums of split apply tiles (items x 32)
-    hssnd::DevBuf d_tickets;     // one ticket counter per split tile
     hssnd::DevBuf apply_buf;     // fronts and work items of every apply stage, one allocation
-    // subtree part of the apply: stages [0, sub_nst) (the deepest levels) run
-    // as one launch per direction, one CTA per subtree rooted in stage
-    // sub_nst - 1; items and per-(subtree, stage) offsets live in apply_buf
-    int sub_nst = 0, sub_n = 0;
-    hssnd::FrontDev *d_sub_fronts = nullptr;
-    hssnd::ApplyItem *d_sub_fwd = nullptr, *d_sub_bwd = nullptr;
-    int *d_sub_off_fwd = nullptr, *d_sub_off_bwd = nullptr;
     // batched factor (hss_factor_batched): device copy of the block-diagonal
     // union of the instances' matrices, used by the batched solver
     int batched = 0;
