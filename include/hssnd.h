@@ -496,6 +496,9 @@ int fgmres_history(int rhs, double *hist, int cap);
  * chunk or pinned staging buffer taken from its scratch pool, every piece of
  * call scratch (device bump allocation or upload staging).  A call that
  * leaves it unchanged allocated nothing.
+ * hss_alloc_fail_next: the nth device allocation that the library makes in the
+ * calling thread from now on (1: the next one) fails with HSS_ENOMEM, once; 0
+ * takes the request back.  Test hook.
  * hss_tc_timeout_selftest: runs one tile of the tensor-core GEMM kernel on an
  * internal 128 x 128 x 32 problem with the MMAs left out, so its bounded
  * mbarrier wait expires after spin_limit polls (1 .. 2^26); returns
@@ -503,6 +506,7 @@ int fgmres_history(int rhs, double *hist, int cap);
  * with nothing left in flight and the context usable.  Test hook. */
 long hss_launch_count(void);
 long hss_alloc_count(void);
+void hss_alloc_fail_next(int nth);
 /* The GEMM engine tuner's process-wide choices (tensor_cores = 3): with
  * idx < 0 the number of shape classes timed so far; otherwise class idx (in
  * the order they were timed): its key (bits 0-11 log2 k, 12-23 log2 n, 24-35

@@ -128,10 +128,18 @@ int current_device() {
 }
 }  // namespace
 
+// Countdown of hss_alloc_fail_next (0: off), of the calling thread only.
+static thread_local int t_fail_in = 0;
+void fail_alloc_in(int nth) { t_fail_in = nth; }
+
 // A cached chunk of at least want bytes, else of at least min; not one so much
 // larger that a later, larger request would miss it; else fresh memory.
 int scratch_cache_take_device(size_t min_bytes, size_t want_bytes, DevBuf &out) {
     count_alloc();
+    if (t_fail_in > 0 && --t_fail_in == 0) {
+        set_error("device allocation of " + std::to_string(want_bytes) + " bytes refused by hss_alloc_fail_next");
+        return HSS_ENOMEM;
+    }
     const int d = current_device();
     const size_t most = std::max(4 * want_bytes, (size_t)64 << 10);
     {
@@ -288,6 +296,8 @@ void Work::reset() {
 extern "C" {
 
 const char *hss_last_error(void) { return hssnd::g_last_error.c_str(); }
+
+void hss_alloc_fail_next(int nth) { hssnd::fail_alloc_in(nth); }
 
 long hss_alloc_count(void) { return hssnd::g_alloc_requests.load(std::memory_order_relaxed); }
 

@@ -218,8 +218,7 @@ static int multi_chunk(int n) { return n < 8192 ? 512 : 1024; }
 template <class T> int pack_apply_multi(hss_factor_t *F, cudaStream_t s) {
     const size_t nst = F->apply.size();
     std::vector<ApplyItem> items;
-    std::vector<ApplyMultiStage> &ms = F->multi;
-    ms.assign(nst, ApplyMultiStage{});
+    std::vector<ApplyMultiStage> ms(nst);
     long part = 0;   // split items of a launch at most: the launches use one buffer in turn
     int tk = 0;
     for (size_t q = 0; q < nst; ++q) {
@@ -260,6 +259,7 @@ template <class T> int pack_apply_multi(hss_factor_t *F, cudaStream_t s) {
         HSS_CUDA(cudaMemcpyAsync(F->multi_items.p, items.data(), sizeof(ApplyItem) * items.size(), cudaMemcpyHostToDevice, s));
     HSS_CUDA(cudaMemsetAsync(F->multi_tickets.p, 0, sizeof(int) * std::max(tk, 1), s));
     // (a copy from pageable memory has left `items` by the time cudaMemcpyAsync returns)
+    F->multi = std::move(ms);   // last: a call after one that failed above packs again
     return HSS_OK;
 }
 
