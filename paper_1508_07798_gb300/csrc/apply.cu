@@ -23,15 +23,27 @@ namespace hssnd {
 
 constexpr int AP_NT = 256;
 constexpr int AP_WPB = AP_NT / 32;   // warps per CTA
-constexpr int APPLY_NCH_MAX = 128;   // chunks of a tile at most: 32 KB of FP64 sums
+constexpr int APPLY_NCH_MAX = 128;   // chunks of a tile at most, one vector: 32 KB of FP64 sums
+// Warps per SM that a level of many tiles is split into, and below which FP64
+// blocks of vectors are split.  24^3 diffusion (fronts to 9,216), FP64, one vector /
+// 8: 16 warps 1,722 / 10,210 us, 32 1,671 / 9,856, 64 1,714 / 10,695, a warp per
+// chunk 1,860 / 14,276; FP32, one vector: 654, 593, 594, 612.
+constexpr int APPLY_WARPS = 32;
+// ... below which FP32 blocks are split: their products are cheap, and a split one
+// reads the factor again (64 x 64 quads, p = 2, 8 vectors: 189 us at most 4, 384 at 32;
+// 16 x 16, p = 1: 64 us never split, 46 split).
+constexpr int APPLY_WARPS_F32 = 4;
+template <class T> constexpr int apply_nv() { return sizeof(T) == 8 ? 4 : 8; }   // vectors of a block at most
+constexpr int APPLY_SUMS = 64 * 1024;   // bytes of a CTA's sums at most in that form
 
-// The products of columns [c0, c1) of a 32-row tile: lane l's sum for row
-// row0 + l.  after_wait() runs once, when the previous kernel's vectors are there.
-template <class T, bool FWD, class AfterWait>
-__device__ __forceinline__ T apply_item_sum(const ApplyItem &it, int c0, int c1, const FrontDev &F,
-                                            const T *__restrict__ arena, const int *__restrict__ iperm,
-                                            const int *__restrict__ blist, const double *w, bool &waited,
-                                            AfterWait &&after_wait) {
+// Adds to acc the products of columns [c0, c1) of a 32-row tile with nv <= NV
+// vectors: lane l's sums for row row0 + l.  after_wait() runs once, when the
+// previous kernel's vectors are there.
+template <class T, bool FWD, int NV, class AfterWait>
+__device__ __forceinline__ void apply_item_sums(const ApplyItem &it, int c0, int c1, const FrontDev &F,
+                                                const T *__restrict__ arena, const int *__restrict__ iperm,
+                                                const int *__restrict__ blist, const double *w, long ldw, int nv,
+                                                bool &waited, AfterWait &&after_wait, T (&acc)[NV]) {
     const int lane = threadIdx.x & 31;
     const T *M = arena + F.foff;
     const int colbase = FWD ? 0 : F.ni, nrows = FWD ? F.n : F.ni;
@@ -39,7 +51,6 @@ __device__ __forceinline__ T apply_item_sum(const ApplyItem &it, int c0, int c1,
     const bool rowok = i < nrows;
     // arithmetic in the factor's precision (FP32 factors: FP32 products and sums;
     // GB300's FP64 pipe is a small fraction of its FP32 rate)
-    T acc = T(0);
     for (int cg = c0; cg < c1; cg += 32) {
         const int c = cg + lane;
         T m[32];
@@ -52,11 +63,28 @@ __device__ __forceinline__ T apply_item_sum(const ApplyItem &it, int c0, int c1,
             waited = true;
             after_wait();
         }
-        const T z = dof >= 0 ? (T)w[dof] : T(0);
+        if constexpr (NV == 1) {
+            const T z = dof >= 0 ? (T)w[dof] : T(0);
 #pragma unroll
-        for (int q = 0; q < 32; ++q) acc = fma(m[q], __shfl_sync(0xffffffffu, z, q), acc);
+            for (int q = 0; q < 32; ++q) acc[0] = fma(m[q], __shfl_sync(0xffffffffu, z, q), acc[0]);
+        } else {
+            T z[NV];
+#pragma unroll
+            for (int r = 0; r < NV; ++r) z[r] = (dof >= 0 && r < nv) ? (T)w[dof + ldw * r] : T(0);
+            // FP64: exactly the vectors there are (a warp's product holds its part of
+            // the FP64 pipe for 64 clocks); FP32: four chains at a time
+            constexpr int G = sizeof(T) == 8 ? 1 : 4;
+#pragma unroll
+            for (int r = 0; r < NV; r += G) {
+                if (r >= nv) break;
+#pragma unroll
+                for (int q = 0; q < 32; ++q)
+#pragma unroll
+                    for (int u = 0; u < G; ++u)
+                        acc[r + u] = fma(m[q], __shfl_sync(0xffffffffu, z[r + u], q), acc[r + u]);
+            }
+        }
     }
-    return acc;
 }
 
 // The dof that lane l of a tile writes (row row0 + l; -1 past the last row), and
@@ -99,39 +127,56 @@ template <class T> __device__ __forceinline__ void store_first_cta(T *p, T v) {
         asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r), "f"(v) : "memory");
 }
 
-// One vector (several: apply_multi.cu).  A 32-row tile of a front is the work of
-// `slots` warps: warp k takes the column chunks k, k + slots, ... of `chunk`
-// columns, lane l owning row row0 + l; x is gathered one value per lane and
-// broadcast by shuffles; 32 matrix loads per lane are in flight before the wait
-// for the previous level.  The warps leave their sums in the shared memory of
-// the tile's (first) CTA, and one warp adds them in chunk order, so the sum order
-// is fixed.  CL = 1: slots <= 8, and a CTA holds 8 / slots tiles; else a cluster
-// of CL CTAs shares one tile.  A level is one chain of latencies (wait, gather,
-// products, sum, store), so partial sums meet in shared memory, not behind a
-// device-wide ticket and a second read (two L2 round trips), and what the store
-// adds to is loaded with the gather.  64 x 64 quads, p = 2, 21 level launches:
-// FP32 (106 MB) 106 -> 71 us, FP64 (208 MB) 197 -> 157 us, of which the FP64 pipe
-// takes 41.  The deepest levels walked by one launch of a CTA per subtree were
-// slower than this kernel's levels (FP32 82, FP64 162 us).
+// NV = 1: one vector; else blocks of up to sh.nv <= NV, sh.ny of them (FP64,
+// and FP32 where apply_multi.cu's tiles are too few, see apply_tiled).  A 32-row
+// tile of a front is the work of `slots` warps: warp k takes the column chunks k,
+// k + slots, ... of `chunk` columns, lane l owning row row0 + l; x is gathered one
+// value per lane and broadcast by shuffles; 32 matrix loads per lane are in flight
+// before the wait for the previous level.  The warps leave their sums in the shared
+// memory of the tile's (first) CTA, and its warps, a vector each, add them in chunk
+// order, so the sum order is fixed.  CL = 1: slots <= 8, and a CTA holds 8 / slots
+// tiles; else a cluster of CL CTAs shares one tile.  A level is one chain of
+// latencies (wait, gather, products, sum, store), so partial sums meet in shared
+// memory, not behind a device-wide ticket and a second read (two L2 round trips),
+// and what the store adds to is loaded with the gather.  64 x 64 quads, p = 2, 22
+// level launches: FP32 (106 MB) 106 -> 71 us, FP64 (208 MB) 197 -> 157 us, of which
+// the FP64 pipe takes 41.  The deepest levels walked by one launch of a CTA per
+// subtree were slower than this kernel's levels (FP32 82, FP64 162 us).
+// Several vectors: FP64 is bound by its pipe (a level of small fronts by the chain
+// of one warp's products: blocks of one or two vectors then), FP32 by the shuffles,
+// one per product and vector.  64 x 64 quads, p = 2, FP64, 3 / 8 / 20 vectors: 355 /
+// 744 / 1,547 us (as tiles of 128 x 512 on one CTA each: 2,896 / 2,891 / 9,355);
+// FP32, 2 / 8 vectors: 131 / 189 us (tiles: 475 / 512).
 //   FWD: y = [F_ii^-1 P^t ; -F_bi F_ii^-1 P^t] x(Iperm)  ->  t = y[0,ni), x_B += y[ni,n)
 //   BWD: x_I = t - W x_B
-template <class T, bool FWD, int CL>
+template <class T, bool FWD, int CL, int NV>
 __global__ void __launch_bounds__(AP_NT) k_apply(const ApplyItem *__restrict__ tiles, int ntiles, ApplyShape sh,
                                                const FrontDev *__restrict__ fr, const T *__restrict__ arena,
                                                const int *__restrict__ iperm, const int *__restrict__ ilist,
                                                const int *__restrict__ blist, const ApplyParams *__restrict__ prm) {
     pdl_launch_next();
     if constexpr (CL > 1) cluster_arrive();
-    extern __shared__ __align__(16) unsigned char apply_smem[];   // [tiles of the CTA][sh.nch][32]
+    extern __shared__ __align__(16) unsigned char apply_smem[];   // [tiles of the CTA][sh.nch][sh.nv][32]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lt = CL > 1 ? 0 : warp / sh.slots;
     const int slot = CL > 1 ? (int)(blockIdx.x % CL) * (int)(blockDim.x / 32) + warp : warp % sh.slots;
-    const int tile = CL > 1 ? (int)(blockIdx.x / CL) : (int)blockIdx.x * sh.per + lt;
-    T *sums = reinterpret_cast<T *>(apply_smem) + (long)lt * sh.nch * 32 + lane;
-    const bool on = tile < ntiles, writer = on && slot == 0;
+    // the blocks of vectors of a tile are neighbours: they read the same factor entries
+    const int g = blockIdx.x / CL, vb = NV == 1 ? 0 : g % sh.ny, tg = NV == 1 ? g : g / sh.ny;
+    const int tile = CL > 1 ? tg : tg * sh.per + lt;
+    T *sums = reinterpret_cast<T *>(apply_smem) + (long)lt * sh.nch * sh.nv * 32 + lane;
+    // the warps that write: of the first CTA, every nw'th vector each
+    const int nw = CL > 1 ? (int)(blockDim.x / 32) : sh.slots;
+    const int nvb = NV == 1 ? 1 : sh.nv, nv = NV == 1 ? 1 : min(nvb, prm->nrhs - nvb * vb);
+    const bool on = tile < ntiles && nv > 0;
+    const bool writer = on && (NV == 1 ? slot == 0 : slot < nw);
     ApplyItem it{};
     FrontDev F{};
+    const long ldw = prm->ldw, ldt = prm->ldt;
     double *w = prm->w, *tv = prm->tv;
+    if constexpr (NV > 1) {
+        w += ldw * nvb * vb;
+        tv += ldt * nvb * vb;
+    }
     int nch = 0, dof = -1;
     if (on) {
         it = tiles[tile];
@@ -139,24 +184,39 @@ __global__ void __launch_bounds__(AP_NT) k_apply(const ApplyItem *__restrict__ t
         nch = max(1, (it.c1 + sh.chunk - 1) / sh.chunk);
         if (writer) dof = apply_dof<FWD>(it, F, ilist, blist);
     }
-    double old = 0.0;
-    T acc = T(0);
+    double old[NV];
+    auto load_old = [&] {   // of the vectors slot, slot + nw, ... in that order
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const int r = NV == 1 ? 0 : slot + nw * k;
+            old[k] = writer && r < nv ? apply_old<FWD>(it, F, dof, w + ldw * r, tv + ldt * r) : 0.0;
+        }
+    };
+    T acc[NV] = {};
     bool waited = false, started = false;
     for (int ch = slot; ch < nch; ch += sh.slots) {
-        acc = apply_item_sum<T, FWD>(it, ch * sh.chunk, min(it.c1, (ch + 1) * sh.chunk), F, arena, iperm, blist, w,
-                                     waited, [&] { old = apply_old<FWD>(it, F, dof, w, tv); });
+#pragma unroll
+        for (int r = 0; r < NV; ++r) acc[r] = T(0);
+        apply_item_sums<T, FWD, NV>(it, ch * sh.chunk, min(it.c1, (ch + 1) * sh.chunk), F, arena, iperm, blist, w, ldw,
+                                    nv, waited, load_old, acc);
         if (sh.nch > 1) {
             if constexpr (CL > 1) {
                 if (!started) cluster_wait();   // the first CTA runs
                 started = true;
-                store_first_cta(sums + ch * 32, acc);
-            } else
-                sums[ch * 32] = acc;
+            }
+#pragma unroll
+            for (int r = 0; r < NV; ++r) {
+                if (r >= nv) break;
+                if constexpr (CL > 1)
+                    store_first_cta(sums + (ch * nvb + r) * 32, acc[r]);
+                else
+                    sums[(ch * nvb + r) * 32] = acc[r];
+            }
         }
     }
     if (!waited) {   // (no columns)
         pdl_wait_prev();
-        old = apply_old<FWD>(it, F, dof, w, tv);
+        load_old();
     }
     if (sh.nch > 1) {
         if constexpr (CL > 1) {
@@ -166,10 +226,21 @@ __global__ void __launch_bounds__(AP_NT) k_apply(const ApplyItem *__restrict__ t
         } else
             __syncthreads();
         if (!writer) return;
-        acc = T(0);
-        for (int ch = 0; ch < nch; ++ch) acc += sums[ch * 32];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const int r = NV == 1 ? 0 : slot + nw * k;
+            if (r >= nv) break;
+            T y = T(0);
+            for (int ch = 0; ch < nch; ++ch) y += sums[(ch * nvb + r) * 32];
+            apply_store<FWD>(it, F, dof, old[k], (double)y, w + ldw * r, tv + ldt * r);
+        }
+    } else if (writer) {   // one chunk: its warp has the sums of every vector (slots = 1, nw = 1)
+#pragma unroll
+        for (int r = 0; r < NV; ++r) {
+            if (r >= nv) break;
+            apply_store<FWD>(it, F, dof, old[r], (double)acc[r], w + ldw * r, tv + ldt * r);
+        }
     }
-    if (writer) apply_store<FWD>(it, F, dof, old, (double)acc, w, tv);
 }
 
 // The arguments for the sweep's kernels, and w = x (every right-hand side)
@@ -186,31 +257,52 @@ __global__ void k_apply_begin(ApplyParams *d, ApplyParams v, long N) {
 
 // How many chunks the widest tile of a level has, and the warps and CTAs a tile
 // gets: a warp per chunk (no idle ones: a level's warps compete for the SMs'
-// registers), up to 8 CTAs of 8 (the portable cluster size).
-static ApplyShape apply_shape(int ncols, int chunk) {
+// registers), up to 8 CTAs of 8 (the portable cluster size); in levels with many
+// tiles only as many as keep APPLY_WARPS warps in flight per SM, at least a CTA's,
+// all doing the same number of chunks.  nch_max: what the sums may take of shared memory.
+static ApplyShape apply_shape(int ntiles, int ncols, int chunk, int nch_max) {
     ApplyShape sh;
     sh.chunk = chunk;
-    while (cdiv(ncols, sh.chunk) > APPLY_NCH_MAX) sh.chunk *= 2;
+    while (cdiv(ncols, sh.chunk) > nch_max) sh.chunk *= 2;
     sh.nch = std::max(1, cdiv(ncols, sh.chunk));
-    while (sh.cl < 8 && sh.nch > sh.cl * AP_WPB) sh.cl *= 2;
-    sh.slots = sh.cl * std::min(AP_WPB, cdiv(sh.nch, sh.cl));
+    const int most = std::min(8 * AP_WPB, std::max(AP_WPB, cdiv(APPLY_WARPS * device_sms(), std::max(ntiles, 1))));
+    const int warps = cdiv(sh.nch, cdiv(sh.nch, most));
+    while (sh.cl < 8 && warps > sh.cl * AP_WPB) sh.cl *= 2;
+    sh.slots = sh.cl * cdiv(warps, sh.cl);
     sh.per = std::max(1, AP_WPB / sh.slots);
     return sh;
 }
 
-template <class T, bool FWD>
-static cudaError_t launch_apply(const hss_factor_t *f, const ApplyStage &st, cudaStream_t s) {
-    const ApplyShape &sh = st.shape[FWD ? 0 : 1];
-    const int nt = FWD ? st.nfwd : st.nbwd;
-    auto kern = sh.cl == 1   ? k_apply<T, FWD, 1>
-                : sh.cl == 2 ? k_apply<T, FWD, 2>
-                : sh.cl == 4 ? k_apply<T, FWD, 4>
-                             : k_apply<T, FWD, 8>;
+// The same for blocks of several vectors, as many per block (a power of two) as
+// leave a level APPLY_WARPS warps per SM.
+template <class T, int NV> static ApplyShape apply_shape_vecs(int ntiles, int ncols, int chunk, int rb) {
+    ApplyShape sh = apply_shape(ntiles, ncols, chunk, APPLY_SUMS / (32 * NV * (int)sizeof(T)));
+    sh.nv = std::min(NV, rb);
+    const long enough = (sizeof(T) == 8 ? APPLY_WARPS : APPLY_WARPS_F32) * (long)device_sms();
+    while (sh.nv > 1 && (long)ntiles * sh.slots * (rb / sh.nv) < enough) sh.nv /= 2;
+    sh.ny = rb / sh.nv;
+    return sh;
+}
+
+// rb: right-hand sides that the launch serves at most
+template <class T, bool FWD, int NV>
+static cudaError_t launch_apply(const hss_factor_t *f, const ApplyStage &st, int rb, cudaStream_t s) {
+    const int pass = FWD ? 0 : 1, nt = FWD ? st.nfwd : st.nbwd;
+    const ApplyShape sh =
+        NV == 1 ? st.shape[pass] : apply_shape_vecs<T, NV>(nt, st.ncols[pass], st.chunk[pass], rb);
+    auto kern = sh.cl == 1   ? k_apply<T, FWD, 1, NV>
+                : sh.cl == 2 ? k_apply<T, FWD, 2, NV>
+                : sh.cl == 4 ? k_apply<T, FWD, 4, NV>
+                             : k_apply<T, FWD, 8, NV>;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cdiv(nt, sh.per) * sh.cl);
+    cfg.gridDim = dim3(cdiv(nt, sh.per) * sh.cl * sh.ny);
     cfg.blockDim = dim3(32 * sh.per * sh.slots / sh.cl);
-    cfg.dynamicSmemBytes = sh.nch > 1 ? sizeof(T) * 32 * sh.nch * sh.per : 0;
+    cfg.dynamicSmemBytes = sh.nch > 1 ? sizeof(T) * 32 * sh.nv * sh.nch * sh.per : 0;
     cfg.stream = s;
+    if (cfg.dynamicSmemBytes > 48 * 1024) {
+        cudaError_t e = func_smem_once((const void *)kern, APPLY_SUMS);
+        if (e != cudaSuccess) return e;
+    }
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_pdl
     at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -229,7 +321,7 @@ static cudaError_t launch_apply(const hss_factor_t *f, const ApplyStage &st, cud
 // The whole sweep (forward levels, top block, backward levels) as one kernel
 // sequence on stream s, each launch overlapping the previous one's tail
 // (launch_pdl); parameters come from f->d_aparams.  RB = 1: one vector; else up
-// to RB.
+// to RB, in the form that each level's launch is better in.
 template <class T, int RB> static int record_sweep(const hss_factor_t *f, cudaStream_t s, int &nk) {
     nk = 0;
     cudaError_t e = cudaSuccess;
@@ -240,10 +332,13 @@ template <class T, int RB> static int record_sweep(const hss_factor_t *f, cudaSt
             const ApplyStage &st = f->apply[q];
             if ((fwd ? st.nfwd : st.nbwd) == 0) continue;
             if (e != cudaSuccess) break;
-            if constexpr (RB > 1)
-                e = launch_apply_multi<T, RB>(f, q, fwd, s);
+            if constexpr (RB == 1)
+                e = fwd ? launch_apply<T, true, 1>(f, st, 1, s) : launch_apply<T, false, 1>(f, st, 1, s);
+            else if (std::is_same<T, float>::value && apply_tiled(st, pass, RB))
+                e = launch_apply_multi<std::max(RB, 8)>(f, q, fwd, s);
             else
-                e = fwd ? launch_apply<T, true>(f, st, s) : launch_apply<T, false>(f, st, s);
+                e = fwd ? launch_apply<T, true, apply_nv<T>()>(f, st, RB, s)
+                        : launch_apply<T, false, apply_nv<T>()>(f, st, RB, s);
             ++nk;
         }
     }
@@ -281,7 +376,8 @@ int pack_apply(hss_factor_t *F, cudaStream_t s) {
     for (size_t q = 0; q < nst; ++q) {
         ApplyStage &st = F->apply[q];
         for (int pass = 0; pass < 2; ++pass) {
-            st.shape[pass] = apply_shape(stage_items(st, pass, items[2 * q + pass]), st.chunk[pass]);
+            st.ncols[pass] = stage_items(st, pass, items[2 * q + pass]);
+            st.shape[pass] = apply_shape((int)items[2 * q + pass].size(), st.ncols[pass], st.chunk[pass], APPLY_NCH_MAX);
             st.chunk[pass] = st.shape[pass].chunk;
         }
         st.nfwd = (int)items[2 * q].size();
@@ -325,7 +421,7 @@ template <class T> static int timed_sweep(const hss_factor_t *f, cudaStream_t s,
             const int nt = fwd ? st.nfwd : st.nbwd;
             if (nt == 0) continue;
             HSS_CUDA(cudaEventRecord(ev[2 * (2 * q + pass)], s));
-            HSS_CUDA((fwd ? launch_apply<T, true>(f, st, s) : launch_apply<T, false>(f, st, s)));
+            HSS_CUDA((fwd ? launch_apply<T, true, 1>(f, st, 1, s) : launch_apply<T, false, 1>(f, st, 1, s)));
             HSS_CUDA(cudaEventRecord(ev[2 * (2 * q + pass) + 1], s));
         }
     }
@@ -429,8 +525,10 @@ template <class T> static int build_graph(hss_factor_t *f, int slot) {
     if (e == cudaSuccess) {
         int nk = 0;
         rc = slot == 0   ? record_sweep<T, 1>(f, cs, nk)
-             : slot == 1 ? record_sweep<T, 8>(f, cs, nk)
-             : slot == 2 ? record_sweep<T, 16>(f, cs, nk)
+             : slot == 1 ? record_sweep<T, 2>(f, cs, nk)
+             : slot == 2 ? record_sweep<T, 4>(f, cs, nk)
+             : slot == 3 ? record_sweep<T, 8>(f, cs, nk)
+             : slot == 4 ? record_sweep<T, 16>(f, cs, nk)
                          : record_sweep<T, 32>(f, cs, nk);
         e = cudaStreamEndCapture(cs, &g);
         f->graph_kernels[slot] = nk;
@@ -449,13 +547,12 @@ int apply_factor(const hss_factor_t *f, int nrhs, const double *x, long ldx, dou
     int rc;
     if ((rc = mf->tvec.alloc(sizeof(double) * (size_t)f->ndof * std::min(nrhs, APPLY_RB)))) return rc;
     if ((rc = mf->d_aparams.alloc(sizeof(ApplyParams)))) return rc;
-    if (nrhs > 1 && f->multi.empty()) {
-        rc = f->precision == HSS_FP32 ? pack_apply_multi<float>(mf, s) : pack_apply_multi<double>(mf, s);
-        if (rc) return rc;
-    }
+    if (nrhs > 1 && f->precision == HSS_FP32 && f->multi.empty() && (rc = pack_apply_multi(mf, s))) return rc;
     HSS_PROF("apply", s, f->apply_bytes(nrhs));
     for (int k = 0; k < nrhs; k += APPLY_RB) {   // one sweep per block of up to APPLY_RB right-hand sides
-        const int nr = std::min(APPLY_RB, nrhs - k), slot = nr == 1 ? 0 : nr <= 8 ? 1 : nr <= 16 ? 2 : 3;
+        const int nr = std::min(APPLY_RB, nrhs - k);
+        int slot = 0;
+        while ((1 << slot) < nr) ++slot;
         if (!f->gexec[slot]) {
             rc = f->precision == HSS_FP32 ? build_graph<float>(mf, slot) : build_graph<double>(mf, slot);
             if (rc) return rc;

@@ -28,7 +28,7 @@ struct ApplyMultiStage {
 // One level launch of the single-vector apply: columns per chunk, the most
 // chunks of a tile, the warps of a tile, and the CTAs of a tile or the tiles of a CTA.
 struct ApplyShape {
-    int chunk = APPLY_CHUNK, nch = 1, slots = 1, cl = 1, per = 1;
+    int chunk = APPLY_CHUNK, nch = 1, slots = 1, cl = 1, per = 1, nv = 1, ny = 1;
 };
 
 // Per level (and the top block): fronts and the row tiles of the apply.
@@ -40,6 +40,7 @@ struct ApplyStage {
     FrontDev *d_fronts = nullptr;
     ApplyItem *d_fwd = nullptr, *d_bwd = nullptr;
     int nfwd = 0, nbwd = 0;               // row tiles of the two sweeps
+    int ncols[2] = {0, 0};                // columns of the widest tile
     ApplyShape shape[2];                  // their warps and CTAs
     double fwd_bytes = 0, bwd_bytes = 0;  // factor entries read (x8 bytes in FP64)
     double fwd_vec = 0, bwd_vec = 0;      // vector entries read + written per right-hand side
@@ -57,10 +58,10 @@ struct ApplyParams {
     int nrhs;
 };
 
-// Right-hand sides per sweep of the apply: 1, or blocks of up to 8, 16 or 32
-// (the factor is read once per sweep).
+// Right-hand sides per sweep of the apply: 1, or blocks of up to 2, 4, .. 32, a
+// captured sweep for each.
 constexpr int APPLY_RB = 32;
-constexpr int APPLY_SLOTS = 4;
+constexpr int APPLY_SLOTS = 6;
 
 struct FrontLog {   // per-front record (rank logging, Sec. 5 empirical cost)
     int box, level, ni, nb, r, rounds, kmax, nnodes;
@@ -74,10 +75,12 @@ int pack_apply(hss_factor_t *F, cudaStream_t s);
 // Chooses each stage's forward and backward column chunk by timing the
 // candidates (process-wide cache keyed by the stage's front shapes).
 int tune_apply(hss_factor_t *F, cudaStream_t s);
-// Several right-hand sides: the work items (at a factor's first such apply) and
-// the launch of one stage and direction.
-template <class T> int pack_apply_multi(hss_factor_t *F, cudaStream_t s);
-template <class T, int RB> cudaError_t launch_apply_multi(const hss_factor_t *F, size_t stage, bool fwd, cudaStream_t s);
+// Several right-hand sides of an FP32 factor as tiled products: whether a level's
+// launch for up to rb of them takes that form, the work items of the levels that
+// can (at a factor's first such apply), and the launch of one stage and direction.
+bool apply_tiled(const ApplyStage &st, int pass, int rb);
+int pack_apply_multi(hss_factor_t *F, cudaStream_t s);
+template <int RB> cudaError_t launch_apply_multi(const hss_factor_t *F, size_t stage, bool fwd, cudaStream_t s);
 int ilu_apply(const hss_ilu_t *M, int nrhs, const double *x, long ldx, double *y, long ldy, cudaStream_t s);
 long ilu_ndof(const hss_ilu_t *M);
 int spmv(const hss_bsr *A, int nrhs, const double *x, long ldx, double *y, long ldy, cudaStream_t s);
@@ -124,7 +127,7 @@ struct hss_factor_t {
     double host_sync_ms = 0;   // host time spent waiting in them
     double host_ms = 0;        // host time of the whole call
     double host_gap_ms = 0;    // host time from each read-back to the next kernel launch (device idle)
-    // captured apply sweeps (slot 0: one right-hand side, 1..3: blocks of 8, 16, 32)
+    // captured apply sweeps (slot k: up to 2^k right-hand sides)
     cudaGraphExec_t gexec[hssnd::APPLY_SLOTS] = {};
     int graph_kernels[hssnd::APPLY_SLOTS] = {};
     std::vector<hssnd::ApplyMultiStage> multi;   // per stage, filled by the first apply to several vectors
