@@ -63,19 +63,11 @@ int DevBuf::alloc(size_t nbytes) {
 }
 
 void DevBuf::release() {
-    if (!p) return;
-    int cur = 0;
-    const bool other = cudaGetDevice(&cur) == cudaSuccess && cur != dev;
-    if (other) cudaSetDevice(dev);
-    if (cudaDeviceSynchronize() == cudaSuccess) {
-        scratch_cache_give_device(std::move(*this));
-    } else {   // (a failed device, or a capture in progress: leave it to the driver)
-        cudaGetLastError();
-        cudaFree(p);
-        forget();
-    }
-    if (other) cudaSetDevice(cur);
+    if (p) cudaFree(p);
+    forget();
 }
+
+void DevBuf::recycle() { scratch_cache_give_device(std::move(*this)); }
 
 // Dynamic shared-memory limit of a kernel, set once per (device, kernel):
 // the attribute belongs to the device context; the set is guarded for calls

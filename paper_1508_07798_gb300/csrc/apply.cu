@@ -590,5 +590,6 @@ extern "C" int hss_apply(const hss_factor_t *f, int nrhs, const double *x, int l
         return HSS_EINVAL;
     }
     if (nrhs == 0) return HSS_OK;
+    f->leave_in_flight();
     return apply_factor(f, nrhs, x, ldx, y, ldy, (cudaStream_t)stream);
 }

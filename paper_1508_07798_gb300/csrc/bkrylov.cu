@@ -403,6 +403,8 @@ int fgmres_lockstep(const hss_bsr *A, const Precond &pc, const std::vector<int> 
         HSS_CHECK_LAUNCH("batched fgmres update");
     }
     HSS_CUDA(cudaStreamSynchronize(s));
+    for (DevBuf *q : {&V, &Z, &w, &r, &part, &H, &cs, &sn, &g, &y, &scal, &est, &act, &jend, &sel, &d_ch, &d_pr})
+        q->recycle();
     bool all = true;
     for (int p = 0; p < P; ++p) {
         const int i = p % ninst;
@@ -430,6 +432,8 @@ extern "C" int fgmres_solve_batched(const hss_factor_t *f, int nrhs, const doubl
         set_error("fgmres_solve_batched: invalid argument (needs a factor from hss_factor_batched; restart in [1, 31])");
         return HSS_EINVAL;
     }
-    return fgmres_lockstep(&f->bA, Precond{f, nullptr}, f->tree->inst_dof, nrhs, b, ldb, x, ldx, o, stats, nullptr,
-                           (cudaStream_t)stream);
+    const int rc = fgmres_lockstep(&f->bA, Precond{f, nullptr}, f->tree->inst_dof, nrhs, b, ldb, x, ldx, o, stats,
+                                   nullptr, (cudaStream_t)stream);
+    if (rc != HSS_OK && rc != HSS_ENOCONV) f->leave_in_flight();
+    return rc;
 }

@@ -1650,6 +1650,7 @@ extern "C" int hss_factor_batched(int ninst, const hss_bsr *As, const hss_tree *
         delete F;
         return rc;
     }
+    F->in_flight = false;
     *out = F;
     return HSS_OK;
 }
@@ -1691,6 +1692,7 @@ extern "C" int hss_factor(const hss_bsr *A, const hss_tree *tree, const hss_fact
         delete F;
         return rc;
     }
+    F->in_flight = false;
     *out = F;
     return HSS_OK;
 }

@@ -148,8 +148,20 @@ struct hss_factor_t {
                  (st.fwd_vec + st.bwd_vec) * 8.0 * nrhs;
         return b + 2.0 * 8.0 * ndof * nrhs;   // copy-in
     }
+    // whether a copy or kernel may still use the buffers: until the factorization is
+    // done, and after calls that return with kernels in flight (hss_apply, or a solve
+    // that failed); the others have waited for theirs
+    mutable std::atomic<bool> in_flight{true};
+    void leave_in_flight() const {
+        in_flight = true;
+        tree->in_flight = true;
+    }
     ~hss_factor_t() {
         for (auto &g : gexec)
             if (g) cudaGraphExecDestroy(g);
+        if (in_flight) return;
+        for (hssnd::DevBuf *b : {&arena, &d_iperm, &d_topset, &tvec, &keep, &multi_items, &multi_tickets, &multi_part,
+                                 &d_aparams, &apply_buf, &b_row, &b_col, &b_val})
+            b->recycle();
     }
 };

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -64,10 +65,11 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     } while (0)
 
 // Device allocation owned by a handle or a call.  Memory comes from the
-// process-wide cache below and goes back to it when the buffer is released,
-// after the device has finished what was launched (the wait that cudaFree
-// implies), so the handles of a program that factors again and again cost no
-// cudaMalloc and cudaFree.
+// process-wide cache below.  release() and the destructor give it to the driver
+// (cudaFree, which waits for whatever may still use it); recycle() gives it back to
+// the cache, for owners that know that nothing does, so the handles of a program
+// that factors and solves again and again cost no cudaMalloc and cudaFree.  No
+// device-wide synchronize: it would break the stream captures of other threads.
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
@@ -92,6 +94,7 @@ struct DevBuf {
         bytes = 0;
     }
     void release();
+    void recycle();
     int alloc(size_t nbytes);  // returns HSS_OK / HSS_ENOMEM
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
@@ -187,6 +190,13 @@ struct hss_tree {
     std::vector<int> iset, bset, fmap, perm, dfs_elem;
     std::vector<std::vector<int>> stages;  // stages[s]: boxes of level maxlev - s (deepest first)
     hssnd::DevBuf d_iset, d_bset, d_fmap;
+    // whether a copy or kernel may still use them: until nd_order has waited for its
+    // own, and after calls that return with kernels in flight (hss_apply)
+    mutable std::atomic<bool> in_flight{true};
+    ~hss_tree() {
+        if (in_flight) return;
+        for (hssnd::DevBuf *b : {&d_iset, &d_bset, &d_fmap}) b->recycle();
+    }
     // HSS tree of each box's S over B^box (nodes in post-order, root last)
     std::vector<std::vector<hssnd::HssNode>> hss;
     // A forest of independent instances (nd_order_batched) concatenates the

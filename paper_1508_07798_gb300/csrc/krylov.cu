@@ -570,7 +570,9 @@ extern "C" int fgmres_solve(const hss_bsr *A, const hss_factor_t *f, int nrhs, c
         set_error("fgmres_solve: invalid argument (restart must be in [1, 31])");
         return HSS_EINVAL;
     }
-    return fgmres_driver(A, Precond{f, nullptr}, nrhs, b, ldb, x, ldx, o, stats, (cudaStream_t)stream);
+    const int rc = fgmres_driver(A, Precond{f, nullptr}, nrhs, b, ldb, x, ldx, o, stats, (cudaStream_t)stream);
+    if (f && rc != HSS_OK && rc != HSS_ENOCONV) f->leave_in_flight();
+    return rc;
 }
 
 extern "C" int fgmres_solve_ilu0(const hss_bsr *A, const hss_ilu_t *M, int nrhs, const double *b, int ldb,

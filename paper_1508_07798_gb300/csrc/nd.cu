@@ -557,6 +557,7 @@ static int nd_order_impl(const hss_mesh *mesh, const hss_bsr *A, const hss_nd_op
     t->box_inst.assign(nbox, 0);
     t->box_local.resize(nbox);
     for (int b = 0; b < nbox; ++b) t->box_local[b] = b;
+    t->in_flight = false;
     *out = t;
     return HSS_OK;
 }
@@ -651,6 +652,7 @@ extern "C" int nd_order_batched(int ninst, const hss_mesh *meshes, const hss_bsr
         delete F;
         return cuda_fail(cudaGetLastError(), "nd_order_batched upload");
     }
+    F->in_flight = false;
     *out = F;
     return HSS_OK;
 }
