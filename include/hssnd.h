@@ -496,6 +496,11 @@ int fgmres_history(int rhs, double *hist, int cap);
  * chunk or pinned staging buffer taken from its scratch pool, every piece of
  * call scratch (device bump allocation or upload staging).  A call that
  * leaves it unchanged allocated nothing.
+ * hss_cache_trim: gives the device and pinned memory that the library keeps for
+ * its next calls and handles (scratch of finished calls, memory of destroyed
+ * handles; at most 8 GB and 512 MB per process) back to the driver, for other
+ * allocators of the process; returns the device bytes given back.  The library
+ * does so itself when one of its own allocations fails.
  * hss_alloc_fail_next: the nth device allocation that the library makes in the
  * calling thread from now on (1: the next one) fails with HSS_ENOMEM, once; 0
  * takes the request back.  Test hook.
@@ -506,6 +511,7 @@ int fgmres_history(int rhs, double *hist, int cap);
  * with nothing left in flight and the context usable.  Test hook. */
 long hss_launch_count(void);
 long hss_alloc_count(void);
+long hss_cache_trim(void);
 void hss_alloc_fail_next(int nth);
 /* The GEMM engine tuner's process-wide choices (tensor_cores = 3): with
  * idx < 0 the number of shape classes timed so far; otherwise class idx (in

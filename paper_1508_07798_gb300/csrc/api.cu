@@ -20,7 +20,7 @@ void count_alloc() { g_alloc_requests.fetch_add(1, std::memory_order_relaxed); }
 
 void set_error(const std::string &msg) { g_last_error = msg; }
 
-static void scratch_cache_trim();
+size_t cache_trim();
 
 int cuda_fail(cudaError_t e, const char *what) {
     g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
@@ -33,7 +33,7 @@ static int raw_alloc(DevBuf &b, size_t nbytes) {
     cudaError_t e = cudaMalloc(&b.p, nbytes);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        scratch_cache_trim();
+        cache_trim();
         e = cudaMalloc(&b.p, nbytes);
     }
     if (e != cudaSuccess) {
@@ -59,7 +59,7 @@ int DevBuf::alloc(size_t nbytes) {
         while (step * 16 <= nbytes) step *= 2;
         want = (nbytes + step - 1) / step * step;
     }
-    return scratch_cache_take_device(nbytes, want, *this);
+    return scratch_cache_take_device(nbytes, want, want + want / 4, *this);   // (held for the owner's life: a close fit)
 }
 
 void DevBuf::release() {
@@ -124,16 +124,16 @@ int current_device() {
 static thread_local int t_fail_in = 0;
 void fail_alloc_in(int nth) { t_fail_in = nth; }
 
-// A cached chunk of at least want bytes, else of at least min; not one so much
-// larger that a later, larger request would miss it; else fresh memory.
-int scratch_cache_take_device(size_t min_bytes, size_t want_bytes, DevBuf &out) {
+// A cached chunk of at least want bytes, else of at least min, and of most bytes or
+// less (but any up to 64 KB); else fresh memory.
+int scratch_cache_take_device(size_t min_bytes, size_t want_bytes, size_t most, DevBuf &out) {
     count_alloc();
     if (t_fail_in > 0 && --t_fail_in == 0) {
         set_error("device allocation of " + std::to_string(want_bytes) + " bytes refused by hss_alloc_fail_next");
         return HSS_ENOMEM;
     }
     const int d = current_device();
-    const size_t most = std::max(4 * want_bytes, (size_t)64 << 10);
+    most = std::max(most, (size_t)64 << 10);
     {
         std::lock_guard<std::mutex> lk(cache().mu);
         auto &v = cache().dev;
@@ -154,33 +154,42 @@ int scratch_cache_take_device(size_t min_bytes, size_t want_bytes, DevBuf &out) 
     return raw_alloc(out, want_bytes);
 }
 
-// Nothing queued on the device may still use b (its caller has waited).
+// Nothing queued on the device may still use b.  Beyond the cache's limit the
+// chunks that have lain in it longest go back to the driver.
 void scratch_cache_give_device(DevBuf &&b) {
     if (!b.p) return;
-    {
+    std::vector<DevBuf> out;   // given back to the driver outside the lock
+    if (b.bytes > CACHE_DEV_MAX) {
+        out.push_back(std::move(b));
+    } else {
         std::lock_guard<std::mutex> lk(cache().mu);
-        if (cache().dev_bytes + b.bytes <= CACHE_DEV_MAX) {
-            cache().dev_bytes += b.bytes;
-            const int d = b.dev;
-            cache().dev.emplace_back(d, std::move(b));
-            return;
+        auto &v = cache().dev;
+        size_t old = 0;
+        while (cache().dev_bytes + b.bytes > CACHE_DEV_MAX) {
+            cache().dev_bytes -= v[old].second.bytes;
+            out.push_back(std::move(v[old++].second));
         }
+        v.erase(v.begin(), v.begin() + old);
+        cache().dev_bytes += b.bytes;
+        const int d = b.dev;
+        v.emplace_back(d, std::move(b));
     }
-    cudaFree(b.p);
-    b.forget();
 }
 
-static void scratch_cache_trim() {
+// Every cached chunk and pinned buffer back to the driver; the device bytes.
+size_t cache_trim() {
     std::vector<std::pair<int, DevBuf>> v;
+    std::vector<std::pair<void *, size_t>> pin;
+    size_t bytes;
     {
         std::lock_guard<std::mutex> lk(cache().mu);
         v.swap(cache().dev);
-        cache().dev_bytes = 0;
+        pin.swap(cache().pin);
+        bytes = cache().dev_bytes;
+        cache().dev_bytes = cache().pin_bytes = 0;
     }
-    for (auto &c : v) {
-        cudaFree(c.second.p);
-        c.second.forget();
-    }
+    for (auto &c : pin) cudaFreeHost(c.first);
+    return bytes;
 }
 
 void *scratch_cache_take_pinned(size_t min_bytes, size_t want_bytes, size_t &got) {
@@ -238,7 +247,7 @@ int Work::dalloc_bytes(size_t bytes, void **out) {
     if (ci >= chunks.size()) {
         size_t want = std::max(bytes, std::max((size_t)(16u << 20), chunks.empty() ? 0 : 2 * chunks.back().bytes));
         DevBuf b;
-        int rc = scratch_cache_take_device(bytes, want, b);
+        int rc = scratch_cache_take_device(bytes, want, 4 * want, b);
         if (rc) return rc;
         chunks.push_back(std::move(b));
         ci = chunks.size() - 1;
@@ -288,6 +297,8 @@ void Work::reset() {
 extern "C" {
 
 const char *hss_last_error(void) { return hssnd::g_last_error.c_str(); }
+
+long hss_cache_trim(void) { return (long)hssnd::cache_trim(); }
 
 void hss_alloc_fail_next(int nth) { hssnd::fail_alloc_in(nth); }
 

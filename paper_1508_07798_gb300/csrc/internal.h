@@ -157,9 +157,9 @@ struct ScratchPtr {
 };
 
 // Process-wide cache of device and pinned memory: thread-safe, at most 8 GB of
-// device memory and 512 MB pinned; a device allocation that fails gives the
-// cached memory back to the driver and tries again.
-int scratch_cache_take_device(size_t min_bytes, size_t want_bytes, DevBuf &out);
+// device memory and 512 MB pinned (the oldest chunks go beyond that); a device
+// allocation that fails, and hss_cache_trim, give all of it back to the driver.
+int scratch_cache_take_device(size_t min_bytes, size_t want_bytes, size_t most, DevBuf &out);
 void scratch_cache_give_device(DevBuf &&b);
 void *scratch_cache_take_pinned(size_t min_bytes, size_t want_bytes, size_t &got);
 void scratch_cache_give_pinned(void *p, size_t bytes);

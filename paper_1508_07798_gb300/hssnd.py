@@ -32,7 +32,7 @@ EXPORTED = [
     "hss_rank_features", "hss_rank_model_create", "hss_rank_model_destroy", "hss_rank_model_get",
     "hss_rank_model_set", "hss_rank_model_fit_norm", "hss_rank_model_loss_grad", "hss_rank_model_train",
     "hss_rank_model_predict", "hss_factor_export_log", "ilu0_factor", "ilu0_apply", "fgmres_solve_ilu0",
-    "ilu0_destroy", "hss_factor_apply_plan", "hss_alloc_count", "hss_alloc_fail_next",
+    "ilu0_destroy", "hss_factor_apply_plan", "hss_alloc_count", "hss_cache_trim", "hss_alloc_fail_next",
     "hss_tc_timeout_selftest",
     "hss_front_eliminate", "hss_front_compress", "hss_gemm_tuner_read",
 ]
@@ -114,6 +114,7 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
         "fgmres_opts_default": (None, [C.POINTER(fgmres_opts)]),
         "hss_launch_count": (C.c_long, []),
         "hss_alloc_count": (C.c_long, []),
+        "hss_cache_trim": (C.c_long, []),
         "hss_alloc_fail_next": (None, [C.c_int]),
         "hss_gemm_tuner_read": (C.c_int, [C.c_int, C.POINTER(C.c_longlong), ip, C.POINTER(C.c_float),
                                           C.POINTER(C.c_float)]),
@@ -583,6 +584,12 @@ def gemm_tuner_choices() -> list:
 def alloc_count() -> int:
     """Memory requests the library has served so far (hss_alloc_count)."""
     return int(_lib.hss_alloc_count())
+
+
+def cache_trim() -> int:
+    """Give the memory the library keeps between calls and of destroyed handles back to
+    the driver (hss_cache_trim); returns the device bytes."""
+    return int(_lib.hss_cache_trim())
 
 
 def alloc_fail_next(nth: int):

@@ -75,3 +75,22 @@ def test_memory_of_a_destroyed_factor_is_not_reused_under_its_apply():
             hs.hss_factor(dA2, hs.nd_order((2, mesh2.n[:2], 2), dA2))
     torch.cuda.synchronize()
     assert torch.equal(y, ref)
+
+
+def test_cached_memory_can_be_given_back_and_small_handles_leave_large_chunks():
+    import torch
+    from paper_1508_07798_gb300 import hssnd as hs
+    mesh, A = dg.diffusion_3d(12, 1, 0)
+    dA = hs.DeviceBSR.from_host(A)
+    tree = hs.nd_order((mesh.dim, mesh.n[:mesh.dim], 1), dA)
+    hs.cache_trim()
+    free0 = torch.cuda.mem_get_info()[0]
+    F = hs.hss_factor(dA, tree, precision="fp64")
+    large = F.info()["factor_bytes"]
+    del F
+    # half its size: the FP32 factor must not sit on the FP64 one's memory
+    F = hs.hss_factor(dA, tree, precision="fp32")
+    assert hs.cache_trim() >= large
+    del F
+    assert hs.cache_trim() > 0 and hs.cache_trim() == 0
+    assert torch.cuda.mem_get_info()[0] >= free0 - (64 << 20)   # (modules loaded meanwhile)
