@@ -887,9 +887,14 @@ int compress_stage(const hss_tree *t, const hss_factor_opts &o, const std::vecto
                     L.r = std::max(L.r, r);
                     L.m = std::max(L.m, m);
                 }
-                const IdClass ic = id_class(L.r, L.m, (int)sizeof(T));
-                L.smem = id_smem_bytes(std::max(L.r, ic.r), L.m, (int)sizeof(T));   // a register form's R has its largest r
                 L.cnt = (int)id_work.size() - L.off;
+                // what the node that needs most takes (widths and columns of different fronts
+                // do not meet in one node); a register form's R has its largest r
+                const IdClass ic = id_class(L.r, L.m, (int)sizeof(T));
+                for (int q = 0; q < L.cnt; ++q) {
+                    const NodeDev &N = nodes[id_work[L.off + q] >> 1];
+                    L.smem = std::max(L.smem, id_smem_bytes(std::max(cfs[N.cf].r, ic.r), N.s[0].mcap, (int)sizeof(T)));
+                }
                 ids.push_back(L);
             }
         }
