@@ -94,8 +94,9 @@ typedef struct hss_factor_opts {
                                brought in by TMA where they are 16-byte aligned with leading dimensions
                                that are multiples of 4 (front sizes divisible by 4), staged by the threads
                                otherwise; 2 tcgen05 with a single TF32 product (threads staging); 3 the
-                               block updates (K >= 128) of fronts of at least 2048 rows as tcgen05 FP16
-                               two-term products (FP32 accuracy like 1, any alignment), and per shape class
+                               block updates (K >= 128) of fronts of at least 2048 rows as tcgen05 products
+                               of three BF16 terms (24 bits of every operand, any alignment; closer to
+                               FP32 arithmetic than 1), and per shape class
                                (operand forms, m, n, k rounded up to powers of two) of the other problems
                                the TMA-fed kernel can take: SIMT or that kernel, timed on a scratch C the
                                first time the class appears (the tensor cores need a 15% lead) and cached

@@ -21,7 +21,7 @@
 #include <cstring>
 
 #include "factor.h"
-#include "h2gemm.h"
+#include "b3gemm.h"
 #include "hss.h"
 #include "prof.h"
 
@@ -103,7 +103,7 @@ template <class T> bool use_tc(const Engine &e, const GemmDesc<T> &d) {
     return std::is_same<T, float>::value && e.tc != 0 && d.m >= 128 && d.n >= 32 && d.k >= 128;
 }
 
-enum { ENG_SIMT = 0, ENG_TMA = 1, ENG_STG = 2, ENG_BF16 = 3, ENG_H2 = 4, NENG = 5 };
+enum { ENG_SIMT = 0, ENG_TMA = 1, ENG_STG = 2, ENG_BF16 = 3, ENG_B3 = 4, NENG = 5 };
 
 // ---- GEMM engine autotuner (tensor_cores = 3): per shape class (operand
 // forms, sizes rounded up to powers of two) of the problems the TMA-fed
@@ -187,12 +187,12 @@ template <class T> int choose_engine(const Engine &E, const GemmDesc<T> &d, Work
             if (use_tc(E, d)) *out = (E.tc == 1 && tma) ? ENG_TMA : ENG_STG;
             return HSS_OK;
         }
-        // tensor_cores = 3: block-end updates as FP16 two-term products.  The split
-        // pass (about 10 us) wants a long contraction and many tiles; against the
-        // TMA-fed kernel, split included: 2048^2 x 256 49 -> 25 us, 4096^2 155 ->
-        // 52, 8192^2 547 -> 142, so every block update qualifies
-        if (d.B && !d.transA && !d.transB && d.k >= 128 && d.k <= H2_KMAX && d.m >= 1024 && d.n >= 1024) {
-            *out = ENG_H2;
+        // tensor_cores = 3: block-end updates as products of three BF16 terms.  The
+        // split pass (about 10 us) wants a long contraction and many tiles; against the
+        // TMA-fed kernel, split included: 2048^2 x 256 49 -> 29 us, 4096^2 155 -> 61,
+        // 8192^2 547 -> 177, so every block update qualifies
+        if (d.B && !d.transA && !d.transB && d.k >= 128 && d.k <= B3_KMAX && d.m >= 1024 && d.n >= 1024) {
+            *out = ENG_B3;
             return HSS_OK;
         }
         // the others: chosen by timing, between SIMT and the TMA-fed kernel
@@ -243,12 +243,12 @@ template <class T> struct GemmPlan {
     std::vector<int> ts;         // tile size of each group's SIMT launch
     TmaGemmDesc *d_tdescs = nullptr;
     GemmTile *d_tl[NENG] = {};
-    // ENG_H2: tiles refer to h2 (the flagged problems only), images shared by the groups
-    std::vector<H2Desc> h2;
-    std::vector<H2Split> split;
+    // ENG_B3: tiles refer to b3 (the flagged problems only), images shared by the groups
+    std::vector<B3Desc> b3;
+    std::vector<B3Split> split;
     std::vector<int> split_off;
-    H2Desc *d_h2 = nullptr;
-    H2Split *d_split = nullptr;
+    B3Desc *d_b3 = nullptr;
+    B3Split *d_split = nullptr;
 };
 
 // Engine of every problem, tiles per (group, engine), uploaded through W.
@@ -272,19 +272,19 @@ int plan_gemms(const Engine &E, const std::vector<GemmDesc<T>> &descs, const std
         P.off[e].assign(ngroups + 1, 0);
         P.fl[e].assign(ngroups, 0.0);
     }
-    P.h2.clear();
+    P.b3.clear();
     P.split.clear();
     P.split_off.assign(ngroups + 1, 0);
-    unsigned char *h2_ws = nullptr;
+    unsigned char *b3_ws = nullptr;
     if constexpr (std::is_same<T, float>::value) {   // the groups run one after another: one group's images at a time
         size_t most = 0;
         for (int g = 0; g < ngroups; ++g) {
             size_t sum = 0;
             for (int i : of[g])
-                if (which[i] == ENG_H2) sum += gemm_h2_bytes(descs[i]);
+                if (which[i] == ENG_B3) sum += gemm_b3_bytes(descs[i]);
             most = std::max(most, sum);
         }
-        if (most && (rc = W.dalloc(most, &h2_ws))) return rc;
+        if (most && (rc = W.dalloc(most, &b3_ws))) return rc;
     }
     P.ts.assign(ngroups, GEMM_TM);
     for (int g = 0; g < ngroups; ++g) {
@@ -294,14 +294,14 @@ int plan_gemms(const Engine &E, const std::vector<GemmDesc<T>> &descs, const std
         P.ts[g] = gemm_tile_size<T>(simt);
         for (int e = 0; e < NENG; ++e) P.off[e][g] = (int)P.tl[e].size();
         P.split_off[g] = (int)P.split.size();
-        size_t h2_off = 0;
+        size_t b3_off = 0;
         for (int i : of[g]) {
             const int e = which[i];
             if constexpr (std::is_same<T, float>::value) {
-                if (e == ENG_H2) {
-                    gemm_h2_desc(descs[i], h2_ws + h2_off, P.h2);
-                    h2_off += gemm_h2_bytes(descs[i]);
-                    gemm_h2_tiles(descs[i], (int)P.h2.size() - 1, P.tl[e], P.split);
+                if (e == ENG_B3) {
+                    gemm_b3_desc(descs[i], b3_ws + b3_off, P.b3);
+                    b3_off += gemm_b3_bytes(descs[i]);
+                    gemm_b3_tiles(descs[i], (int)P.b3.size() - 1, P.tl[e], P.split);
                     P.fl[e][g] += gemm_flops(descs[i]);
                     continue;
                 }
@@ -321,7 +321,7 @@ int plan_gemms(const Engine &E, const std::vector<GemmDesc<T>> &descs, const std
         if ((!P.tl[ENG_TMA].empty() || !P.tl[ENG_BF16].empty()) &&
             (rc = gemm_tma_descs(descs, use_tma, W, &P.d_tdescs)))
             return rc;
-        if (!P.h2.empty() && ((rc = W.up(P.h2, &P.d_h2)) || (rc = W.up(P.split, &P.d_split)))) return rc;
+        if (!P.b3.empty() && ((rc = W.up(P.b3, &P.d_b3)) || (rc = W.up(P.split, &P.d_split)))) return rc;
     }
     return HSS_OK;
 }
@@ -344,8 +344,8 @@ int run_gemm_group(const Engine &E, const GemmPlan<T> &P, const GemmDesc<T> *d_d
                 return HSS_ECUDA;
             }
             if (e == ENG_TMA) rc = gemm_tma(P.d_tdescs, t, n, E.err, s, P.fl[e][g], tma_class);
-            else if (e == ENG_H2)
-                rc = gemm_h2(P.d_h2, P.d_split + P.split_off[g], P.split_off[g + 1] - P.split_off[g], t, n, E.err, s,
+            else if (e == ENG_B3)
+                rc = gemm_b3(P.d_b3, P.d_split + P.split_off[g], P.split_off[g + 1] - P.split_off[g], t, n, E.err, s,
                              P.fl[e][g], tma_class);
             else if (e == ENG_BF16) rc = gemm_tma(P.d_tdescs, t, n, E.err, s, P.fl[e][g], "gemm_bf16_sample", true);
             else rc = gemm_tc(d_descs, t, n, E.tc == 2 ? 0 : 1, E.err, s, P.fl[e][g]);
@@ -1404,7 +1404,7 @@ template <class T> int factor_impl(const hss_bsr *A, const hss_tree *t, const hs
             }
         if (eng.tc && (rc = check_tc())) return rc;
         F->gemm_simt = eng.problems[ENG_SIMT];
-        F->gemm_tma = eng.problems[ENG_TMA] + eng.problems[ENG_H2];
+        F->gemm_tma = eng.problems[ENG_TMA] + eng.problems[ENG_B3];
         F->gemm_staged = eng.problems[ENG_STG];
         F->gemm_timed = eng.timed;
         F->gemm_bf16 = eng.problems[ENG_BF16];
