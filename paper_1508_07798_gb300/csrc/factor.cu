@@ -377,7 +377,7 @@ int eliminate_stage(const std::vector<FrontDev> &fr, const FrontDev *d_fr, T *ar
     HSS_HOST("eliminate_stage");
     int nf = (int)fr.size();
     const bool phased = pbeg != nullptr;
-    std::vector<int> kb(nf), nsteps(nf), isreg(nf), Rf(nf), clpath(nf, 0), beg(nf), end(nf);
+    std::vector<int> kb(nf), nsteps(nf), isreg(nf), Rf(nf), clpath(nf, 0), beg(nf), end(nf), npb(nf, PANEL_BLOCK);
     std::vector<long> aoff(nf);
     long aold_total = 0;
     int maxsteps = 0;
@@ -393,6 +393,14 @@ int eliminate_stage(const std::vector<FrontDev> &fr, const FrontDev *d_fr, T *ar
         // tall fronts: 32-column panels spread over a cluster while their rows
         // exceed one CTA's registers, then the register panel
         if (fr[f].ni > (sizeof(T) == 4 ? PANEL_CL_MIN_NI_F32 : PANEL_CL_MIN_NI) && panel_cl_fits(PANEL_KB_MAX, fr[f].ni, (int)sizeof(T))) {
+            // a block as wide as with register panels of this height: its width decides
+            // the rounding of its explicit inverse; 128 pivots at least where the
+            // three-term products take the updates.  W of decaying, one-sign and
+            // row-scaled fronts of 1,600 to 6,100 pivots with 256 everywhere: 1.3 to 2
+            // times the error in FP32 arithmetic (tensor_cores 0); so: 1.0 to 1.2, with
+            // tensor_cores 3 0.2 to 0.7 of the TF32 split's in blocks of that width.
+            // 32^3 diffusion 532 -> 553 ms.
+            if (isreg[f]) npb[f] = std::max(eng.tc == 3 ? 4 : 2, PANEL_BLOCK * kb[f] / PANEL_KB_MAX);
             kb[f] = PANEL_KB_MAX;
             isreg[f] = 0;
             clpath[f] = 1;
@@ -412,7 +420,7 @@ int eliminate_stage(const std::vector<FrontDev> &fr, const FrontDev *d_fr, T *ar
         size_t smem;
         double flops;   // algorithmic work of the group's panels: 2 hT kb^2 each
     };
-    // Large fronts (n >= PANEL_BLOCK_MIN_N) run in blocks of PANEL_BLOCK
+    // Large fronts (n >= PANEL_BLOCK_MIN_N) run in blocks of up to PANEL_BLOCK
     // panels: a panel's row moves and update reach only the columns of its
     // block; at the end of a block the other columns take the block's row
     // moves and one update of the block's width (for Gauss-Jordan,
@@ -426,7 +434,7 @@ int eliminate_stage(const std::vector<FrontDev> &fr, const FrontDev *d_fr, T *ar
     long aoldB_total = 0;
     for (int f = 0; f < nf; ++f) {
         aoffB[f] = aoldB_total;
-        aoldB_total += (long)PANEL_BLOCK * kb[f] * fr[f].n;
+        aoldB_total += (long)npb[f] * kb[f] * fr[f].n;
     }
     std::vector<PanelJob> jobs;
     std::vector<std::vector<int>> jobs_of(nf);
@@ -486,8 +494,8 @@ int eliminate_stage(const std::vector<FrontDev> &fr, const FrontDev *d_fr, T *ar
             // fronts below PANEL_BLOCK_MIN_N (and phased sweeps): one block
             // spanning every column (the plain per-panel update)
             const bool blocked = n >= PANEL_BLOCK_MIN_N && !phased;
-            const int K0 = blocked ? (st / PANEL_BLOCK) * PANEL_BLOCK * kb[f] : 0;
-            const int bw = blocked ? std::min(PANEL_BLOCK * kb[f], fr[f].ni - K0) : n;
+            const int K0 = blocked ? (st / npb[f]) * npb[f] * kb[f] : 0;
+            const int bw = blocked ? std::min(npb[f] * kb[f], fr[f].ni - K0) : n;
             size_t hT = (size_t)(fr[f].ni - k0);
             int use_smem = 0;
             size_t need = 0;
@@ -537,13 +545,13 @@ int eliminate_stage(const std::vector<FrontDev> &fr, const FrontDev *d_fr, T *ar
             d.skip_hi = k0 - K0 + kbs;
             if (bw > kbs) add_desc(d, aoff[f] + (long)kbs * K0, false, 2 * st);
             // end of the block: the other columns
-            const bool block_end = blocked && ((st % PANEL_BLOCK == PANEL_BLOCK - 1) || st == nsteps[f] - 1);
+            const bool block_end = blocked && ((st % npb[f] == npb[f] - 1) || st == nsteps[f] - 1);
             if (block_end && n > bw) {
                 BlockJob bj{};
                 bj.front = f;
                 bj.k0 = K0;
                 bj.width = bw;
-                bj.np = st % PANEL_BLOCK + 1;
+                bj.np = st % npb[f] + 1;
                 for (int q = 0; q < bj.np; ++q) bj.job[q] = jobs_of[f][st - bj.np + 1 + q];
                 bj.aoff = aoffB[f];
                 const int bjid = (int)bjobs.size();
