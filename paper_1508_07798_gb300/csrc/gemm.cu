@@ -191,6 +191,10 @@ __global__ void __launch_bounds__(gemm_nt<T, TS>(), GemmCfg<T, TS>::CTAS)
 template <class T>
 int gemm_batched(const GemmDesc<T> *d_desc, const GemmTile *d_tiles, int ntiles, cudaStream_t s, double flops, int ts) {
     if (ntiles <= 0) return HSS_OK;
+    if (ts != 32 && !(ts == 64 && sizeof(T) == 4)) {
+        set_error("gemm_batched: no kernel for tiles of " + std::to_string(ts));
+        return HSS_EINVAL;
+    }
     HSS_PROF(sizeof(T) == 8 ? "gemm_f64" : "gemm_f32", s, flops);
     if (ts == 32)
         HSS_CUDA(launch_pdl(k_gemm<T, 32>, dim3(ntiles), dim3(gemm_nt<T, 32>()), 0, s, d_desc, d_tiles));

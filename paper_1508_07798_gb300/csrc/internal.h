@@ -252,10 +252,9 @@ constexpr int GEMM_TN = 64;
 constexpr int GEMM_TC_TM = 128;   // tile of the tcgen05 GEMM (one MMA M x N)
 constexpr int GEMM_TC_TN = 128;
 
-// ts: the tile size (64 or 32) the list was made for
+// ts: the tile size the list was made for (gemm_tile_size; 64 or 32, FP64 32 only)
 template <class T>
-int gemm_batched(const GemmDesc<T> *d_desc, const GemmTile *d_tiles, int ntiles, cudaStream_t s,
-                 double flops = 0.0, int ts = GEMM_TM);
+int gemm_batched(const GemmDesc<T> *d_desc, const GemmTile *d_tiles, int ntiles, cudaStream_t s, double flops, int ts);
 // Tile size of a launch of these problems: 32 below so many 64 x 64 tiles (about
 // one and a half waves of them: launches of 36 to 1,000 tiles are most of a
 // factorization's; limits of 600 and 2,000 measured alike, always 64 cost the 64 x
@@ -301,7 +300,7 @@ template <class T> double gemm_flops(const GemmDesc<T> &d) {
 }
 
 template <class T>
-void gemm_tiles_for(const GemmDesc<T> &d, int desc_index, std::vector<GemmTile> &tiles, int ts = GEMM_TM);
+void gemm_tiles_for(const GemmDesc<T> &d, int desc_index, std::vector<GemmTile> &tiles, int ts);
 
 // ---------------------------------------------------------------- device helpers
 __host__ __device__ inline uint64_t splitmix64(uint64_t x) {

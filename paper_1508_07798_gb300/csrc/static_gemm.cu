@@ -133,7 +133,7 @@ extern "C" int hss_gemm_f32_static(int m, int n, int k, const float *A, int lda,
         HSS_CHECK_LAUNCH("k_gemm_static_setup");
     }
     if (engine == 0)
-        rc = gemm_batched<float>(dd, dt, ntiles, s, 2.0 * m * n * k);
+        rc = gemm_batched<float>(dd, dt, ntiles, s, 2.0 * m * n * k, GEMM_TM);
     else
         rc = gemm_tc(dd, dt, ntiles, engine == 1 ? 1 : 0, err, s, 2.0 * m * n * k);
     if (rc) return rc;

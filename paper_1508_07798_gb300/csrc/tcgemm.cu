@@ -316,8 +316,9 @@ extern "C" int hss_gemm_f32(int m, int n, int k, const float *A, int lda, const 
     d.beta = beta;
     if (engine == 3 && !gemm_tma_eligible(d)) engine = 1;   // operands TMA cannot address
     std::vector<GemmTile> tiles;
+    const int ts = gemm_tile_size<float>({&d});
     if (engine == 0)
-        gemm_tiles_for(d, 0, tiles);
+        gemm_tiles_for(d, 0, tiles, ts);
     else
         gemm_tc_tiles_for(d, 0, tiles);
     Work W(s);
@@ -329,7 +330,7 @@ extern "C" int hss_gemm_f32(int m, int n, int k, const float *A, int lda, const 
     if ((rc = W.up(dv, &dd)) || (rc = W.up(tiles, &dt)) || (rc = W.dalloc(1, &err))) return rc;
     HSS_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     if (engine == 0) {
-        rc = gemm_batched<float>(dd, dt, (int)tiles.size(), s, 2.0 * m * n * k);
+        rc = gemm_batched<float>(dd, dt, (int)tiles.size(), s, 2.0 * m * n * k, ts);
     } else if (engine == 3) {
         TmaGemmDesc *td;
         if ((rc = gemm_tma_descs(dv, std::vector<char>{1}, W, &td))) return rc;
