@@ -11,10 +11,10 @@
 // the factor again for every 8 and gathers x for every 32 rows.  An item is a
 // serial chain of chunks on one CTA, so only levels with items for every SM run
 // here (apply_tiled); FP64 never does: two FMAs per clock and SM make an item of
-// 128 x 512 x 8 products 0.13 ms.  Sums run over segments of `seg` columns, then
+// 128 x 256 x 8 products 66 us.  Sums run over segments of `seg` columns, then
 // over the segments and the items of a row in order (the last CTA to finish adds
-// the items): up to 512 columns the order of k_apply, whose chunks the segments are.
-// 20 vectors, 32^3 diffusion (8.5 GB): 12.6 -> 5.0 ms per apply, bound by the
+// the items): up to 256 columns the order of k_apply, whose chunks the segments are.
+// 20 vectors, 32^3 diffusion (8.5 GB): 12.6 -> 5.3 ms per apply, bound by the
 // shared-memory loads of the products (three of 16 bytes per 32 FMAs).
 #include <algorithm>
 #include <cstring>
@@ -201,10 +201,12 @@ __global__ void __launch_bounds__(MA_NT) k_apply_multi(const ApplyItem *__restri
     }
 }
 
-// Columns per item of a front of order n: a split row tile writes and reads 128
-// x RB partial sums per item (16 KB against 256 KB of the factor at 512 columns).
-// By the front alone, so that a forest sums as its instances do.
-static int multi_chunk(int n) { return n < 8192 ? 512 : 1024; }
+// Columns per item: a split row tile writes and reads 128 x RB partial sums per
+// item (16 KB against 128 KB of the factor), a long item is a long chain.  ms per
+// apply of 20 vectors with 128 / 192 / 256 / 384 / 512 / 1,024 columns: 16^3 diffusion
+// 0.66, 0.67, 0.71, 0.86, 0.99, 1.44; 24^3 2.14, 2.02, 1.97, 2.02, 2.07, 2.56; 32^3 5.9,
+// 5.5, 5.3, 5.2, 5.2, 5.6; 32 vectors, 24 instances: 2.2, 2.2, 2.2, 2.2, 2.3.
+constexpr int MA_COLS = 256;
 
 // Levels with this many products (factor entries times vectors) or more take the
 // tiles.  Launches of seven factors (2D p = 2, 3 to 128 x 128, 3D to 24^3), all with
@@ -233,7 +235,7 @@ int pack_apply_multi(hss_factor_t *F, cudaStream_t s) {
                 const FrontDev &d = st.h_fronts[f];
                 if (d.ni == 0) continue;
                 const int nrows = pass == 0 ? d.n : d.ni, ncols = pass == 0 ? d.ni : d.nb;
-                const int chunk = multi_chunk(d.n), nch = std::max(1, cdiv(ncols, chunk));
+                const int chunk = MA_COLS, nch = std::max(1, cdiv(ncols, chunk));
                 for (int r0 = 0; r0 < nrows; r0 += MA_ROWS) {
                     for (int ch = 0; ch < nch; ++ch) {
                         ApplyItem it{f, r0, std::min(ncols, ch * chunk), std::min(ncols, (ch + 1) * chunk), -1, first, nch};
