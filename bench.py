@@ -122,10 +122,11 @@ def roofline_of(kernel, ms, cnt, work, total_ms, pk, workload=None):
     per_launch_s = ms / cnt * 1e-3
     if kernel == "gemm_tma_block":
         # the blocked sweep's K = 256 updates C += A B of whole fronts on the tensor cores
-        # (tensor_cores = 3: products of three BF16 terms, 1: the TMA-fed TF32 split): at K = 256 their arithmetic intensity against the C stream (read + write, 8 B per
+        # (tensor_cores = 3: products of three BF16 terms, 1: the TMA-fed TF32 split): at
+        # K = 256 their arithmetic intensity against the C stream (read + write, 8 B per
         # output; A and B come from L2) is 2 * 256 / 8 = 64 flop/B, below the TF32 ridge, so HBM
-        # bounds them: algorithmic bytes = flops / 64 (ragged last blocks have K < 256: an
-        # underestimate of their bytes)
+        # bounds them: algorithmic bytes = flops / 64 (ragged last blocks, and fronts of 1,537
+        # to 6,144 interior dofs, have K < 256: an underestimate of their bytes)
         tflops = work / cnt / per_launch_s / 1e12
         ach = work / 64.0 / cnt / per_launch_s / 1e9
         return dict(kernel=kernel, bound="hbm", achieved=ach, peak=pk["hbm"], unit="GB/s", frac=ach / pk["hbm"],

@@ -87,8 +87,9 @@ int panel_cl_capacity(int rows, int tsize);
 // Fronts with more interior dofs take the cluster panel.  FP32: where 32-column
 // panels leave one CTA's registers; the narrower register panels beyond took 2 to
 // 4 times the panel, post-panel and update launches and blocks of 128 or 64
-// columns (a 6,000-row front with 4,000 interior dofs: panels 8.6 -> 7.8, post
-// 5.0 -> 1.7, in-block updates 4.2 -> 1.6, block updates 8.2 -> 1.5 ms).
+// columns (a 6,000-row front with 4,000 interior dofs, tensor_cores 3: panels 8.3 ->
+// 7.9, post 4.4 -> 1.9, in-block updates 4.1 -> 1.1, block updates 8.2 -> 2.8 ms; the
+// blocks keep 64 or 128 pivots, see eliminate_stage).
 // FP64: beyond 6,144, where the register panels end.
 constexpr int PANEL_CL_MIN_NI = 6144, PANEL_CL_MIN_NI_F32 = 1536;
 template <class T>
