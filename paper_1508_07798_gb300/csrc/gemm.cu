@@ -279,6 +279,7 @@ int gemm_f32_k0(float *C, int ldc, int m, int n, float alpha, float beta, cudaSt
 int gemm_f32_prepare() {
     cudaFuncAttributes fa;
     HSS_CUDA(cudaFuncGetAttributes(&fa, k_gemm<float, 64>));
+    HSS_CUDA(cudaFuncGetAttributes(&fa, k_gemm<float, 32>));
     HSS_CUDA(cudaFuncGetAttributes(&fa, k_gemm_k0));
     return HSS_OK;
 }

@@ -261,6 +261,12 @@ int gemm_batched(const GemmDesc<T> *d_desc, const GemmTile *d_tiles, int ntiles,
 // 64, p = 2 factorization 0.8 ms, always 32 the p = 3 one 0.4 ms).
 template <class T> int gemm_tile_size(const std::vector<const GemmDesc<T> *> &group);
 constexpr long GEMM_SMALL_LIMIT = 2000;
+// The tile of one FP32 problem by itself, of any K (hss_gemm_f32): 64 from 1,000 of
+// them on.  64 against 32, us: 64^3 16, 8; 512^3 53, 26; 4,096 x 64 x 4,096 357, 164;
+// 1,024^3 100, 104; 2,048^2 x 32 19.1, 19.7; x 256 81, 91; 2,048^3 560, 670.
+inline int gemm_single_tile(int m, int n) {
+    return (long)((m + 63) / 64) * ((n + 63) / 64) < 1000 ? 32 : 64;
+}
 int launch_sign_bits(const SignBlock *d_blocks, int nblocks, uint64_t seed, uint32_t *out, cudaStream_t s);
 
 // Tensor-core (tcgen05, TF32) GEMM of the FP32 form: split = 1 uses the

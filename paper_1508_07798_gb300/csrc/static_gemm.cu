@@ -94,7 +94,7 @@ extern "C" int hss_gemm_f32_static(int m, int n, int k, const float *A, int lda,
         return HSS_EINVAL;
     }
     if (m == 0 || n == 0) return HSS_OK;
-    const int tile_m = engine == 0 ? GEMM_TM : GEMM_TC_TM, tile_n = engine == 0 ? GEMM_TN : GEMM_TC_TN;
+    const int tile_m = engine == 0 ? gemm_single_tile(m, n) : GEMM_TC_TM, tile_n = engine == 0 ? tile_m : GEMM_TC_TN;
     const long tm = cdiv(m, tile_m), tn = cdiv(n, tile_n);
     if (k > 0 && tm * tn > HSS_GEMM_STATIC_MAX_TILES) {   // (k = 0 needs no tile records)
         set_error("hss_gemm_f32_static: " + std::to_string(m) + " x " + std::to_string(n) + " needs " +
@@ -133,7 +133,7 @@ extern "C" int hss_gemm_f32_static(int m, int n, int k, const float *A, int lda,
         HSS_CHECK_LAUNCH("k_gemm_static_setup");
     }
     if (engine == 0)
-        rc = gemm_batched<float>(dd, dt, ntiles, s, 2.0 * m * n * k, GEMM_TM);
+        rc = gemm_batched<float>(dd, dt, ntiles, s, 2.0 * m * n * k, tile_m);
     else
         rc = gemm_tc(dd, dt, ntiles, engine == 1 ? 1 : 0, err, s, 2.0 * m * n * k);
     if (rc) return rc;

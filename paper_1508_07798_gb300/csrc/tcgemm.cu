@@ -316,7 +316,7 @@ extern "C" int hss_gemm_f32(int m, int n, int k, const float *A, int lda, const 
     d.beta = beta;
     if (engine == 3 && !gemm_tma_eligible(d)) engine = 1;   // operands TMA cannot address
     std::vector<GemmTile> tiles;
-    const int ts = gemm_tile_size<float>({&d});
+    const int ts = gemm_single_tile(m, n);
     if (engine == 0)
         gemm_tiles_for(d, 0, tiles, ts);
     else

@@ -1,17 +1,14 @@
-"""Both tiles of the FP32 SIMT GEMM (32 x 32: hss_gemm_f32 below 2,000 tiles of 64,
-as the launches of a factorization; 64 x 64: hss_gemm_f32_static, and hss_gemm_f32
-above) at the edges of the tiles and of the three-stage ring of K chunks of 16.
-Both add the products in order of K, so they agree bit for bit."""
+"""Both tiles of the FP32 SIMT GEMM (hss_gemm_f32 and hss_gemm_f32_static: 32 x 32
+below 1,000 tiles of 64, else 64 x 64) at the edges of the tiles and of the
+three-stage ring of K chunks of 16.  Both add the products in order of K, so they
+agree bit for bit."""
 import pytest
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (31, 33, 15), (32, 32, 16), (33, 31, 17), (63, 65, 31), (64, 64, 32),
-                                   (65, 63, 33), (95, 97, 47), (96, 96, 48), (97, 95, 49), (200, 7, 64), (7, 200, 65)])
-def test_both_tiles_at_their_edges(m, n, k):
+def _data(m, n, k):
     import torch
-    from paper_1508_07798_gb300 import hssnd as hs
     g = torch.Generator(device="cuda").manual_seed(m * n + k)
     A = torch.randn(m, k, device="cuda", generator=g)
     B = torch.randn(k, n, device="cuda", generator=g)
@@ -19,22 +16,31 @@ def test_both_tiles_at_their_edges(m, n, k):
     ref = 0.5 * (A.double() @ B.double()) - 2.0 * C.double()
     # k products and a sum, each rounded once: (k + 3) u relative to the terms
     bound = (k + 3) * 6e-8 * (0.5 * A.abs().double() @ B.abs().double() + 2.0 * C.abs().double()) + 1e-30
-    small = hs.gemm_f32(A, B, C.clone(), alpha=0.5, beta=-2.0, engine=0)
-    large = C.clone()
-    hs.gemm_f32_static(A, B, large, alpha=0.5, beta=-2.0, engine=0)
-    assert torch.all((small.double() - ref).abs() <= bound)
-    assert torch.equal(small.cpu(), large.cpu())
+    return A, B, C, ref, bound
 
 
-@pytest.mark.parametrize("k", [15, 49])
-def test_large_launch_takes_the_large_tile_with_the_same_sums(k):
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (31, 33, 15), (32, 32, 16), (33, 31, 17), (63, 65, 31), (64, 64, 32),
+                                   (65, 63, 33), (95, 97, 47), (96, 96, 48), (97, 95, 49), (200, 7, 64), (7, 200, 65)])
+def test_small_tile_at_its_edges(m, n, k):
     import torch
     from paper_1508_07798_gb300 import hssnd as hs
-    m, n = 2881, 2945   # 46 x 47 tiles of 64, ragged on both sides
-    g = torch.Generator(device="cuda").manual_seed(k)
-    A = torch.randn(m, k, device="cuda", generator=g)
-    B = torch.randn(k, n, device="cuda", generator=g)
-    C = torch.randn(m, n, device="cuda", generator=g)
-    whole = hs.gemm_f32(A, B, C.clone(), engine=0)
-    part = hs.gemm_f32(A[:1000].contiguous(), B, C[:1000].clone(), engine=0)
-    assert torch.equal(whole[:1000].cpu(), part.cpu())
+    A, B, C, ref, bound = _data(m, n, k)
+    out = hs.gemm_f32(A, B, C.clone(), alpha=0.5, beta=-2.0, engine=0)
+    fixed = C.clone()
+    hs.gemm_f32_static(A, B, fixed, alpha=0.5, beta=-2.0, engine=0)
+    assert torch.all((out.double() - ref).abs() <= bound)
+    assert torch.equal(out, fixed)
+
+
+@pytest.mark.parametrize("k", [1, 15, 16, 17, 31, 32, 33, 47, 48, 49])
+def test_large_tile_at_its_edges_with_the_sums_of_the_small_one(k):
+    import torch
+    from paper_1508_07798_gb300 import hssnd as hs
+    A, B, C, ref, bound = _data(2881, 2945, k)   # 46 x 47 tiles of 64, one row and one column over
+    out = hs.gemm_f32(A, B, C.clone(), alpha=0.5, beta=-2.0, engine=0)
+    fixed = C.clone()
+    hs.gemm_f32_static(A, B, fixed, alpha=0.5, beta=-2.0, engine=0)
+    assert torch.all((out.double() - ref).abs() <= bound)
+    assert torch.equal(out, fixed)
+    part = hs.gemm_f32(A[2000:].contiguous(), B, C[2000:].clone(), alpha=0.5, beta=-2.0, engine=0)   # 14 x 47: the small one
+    assert torch.equal(out[2000:], part)
